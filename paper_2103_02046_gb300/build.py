@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libp3m.so")
-SOURCES = ["ctx.cu", "sort.cu", "pm.cu", "zconv.cu", "zsolve_df.cu", "box.cu", "pp.cu",
+SOURCES = ["ctx.cu", "sort.cu", "pm.cu", "zconv.cu", "zsolve_df.cu", "box.cu", "pp.cu", "pp64.cu",
            "particles.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -35,8 +35,8 @@ def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
     t = os.path.getmtime(obj)
-    deps = [src, os.path.join(CSRC, "p3m_internal.cuh"), os.path.join(CSRC, "df_math.cuh"),
-            os.path.join(ROOT, "include", "p3m.h")]
+    deps = [src, os.path.join(ROOT, "include", "p3m.h")]
+    deps += [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 

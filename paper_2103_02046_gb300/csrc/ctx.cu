@@ -109,6 +109,14 @@ Geom make_geom(const p3m_params* p, int64_t n_max) {
     ext_max = std::max(ext_max, ext[d]);
   }
   g.slack = std::max(1e-4, 1e-6 * ext_max);
+  {
+    int E = 1;  // every position, and every image within reach of one, lies below 2^E
+    while (std::ldexp(1.0, E) < ext_max + 2.0) ++E;
+    g.pos_scale = std::ldexp(1.0, 56 - E);
+    g.pos_hs = static_cast<float>(std::ldexp(1.0, E - 24));
+    g.pos_ms = static_cast<float>(std::ldexp(1.0, E - 48));
+    g.pos_ls = static_cast<float>(std::ldexp(1.0, E - 56));
+  }
   const double cap = std::max<double>(4.0 * static_cast<double>(n_max), 1 << 20);
   auto layout = [&](int rows, int nsub) {
     g.rows = rows;
@@ -275,7 +283,7 @@ cudaError_t alloc(T** ptr, size_t count) {
 
 void free_all(p3m_ctx* c) {
   void* bufs[] = {c->counts, c->starts, c->bsum, c->keys, c->ranks, c->recp, c->recm, c->fpp,
-                  c->fplo, c->pdf,
+                  c->fplo, c->pdf, c->ptab, c->wbound,
                   c->acc, c->qpad, c->qhat, c->qhat2, c->khat_f, c->khat_i, c->fhat, c->freal,
                   c->phihat, c->phireal, c->dfac, c->ztw, c->box_real, c->box_spec, c->box_mult,
                   c->energy_acc, c->pair_acc,
@@ -655,7 +663,9 @@ p3m_status p3m_create(const p3m_params* params, int64_t n_max, void* stream, p3m
       if (e == cudaSuccess)
         e = cudaMemcpy(c->pdf, tab.get(), sizeof(dfm::PairDF), cudaMemcpyHostToDevice);
     }
+    if (e == cudaSuccess) e = pair_table_setup(c);
   }
+  if (!c->fp32) A(alloc(&c->wbound, 1));
   if (params->adj_slots > 0) {
     A(alloc(&c->ckpt, static_cast<size_t>(params->adj_slots) * 6 * n_max));
     A(alloc(&c->seg, static_cast<size_t>(params->adj_segment + 1) * 3 * n_max));

@@ -29,6 +29,7 @@
 
 namespace dfm {
 struct PairDF;
+struct PairTab;
 }
 
 namespace p3m {
@@ -71,6 +72,10 @@ struct Geom {
   float inv_h_df[3][2];  // 1 / h_d
   float fscale_f[3];     // -q / h_d in FP32
   float rch_df[3][2];    // r_c / h_d: cutoff units -> mesh units
+  // FP64 path: positions in cutoff units as 56-bit fixed point below 2^E (E: the mesh extent),
+  // split into 24 + 24 + 8 bits: the units of the pieces and the number of units in 1
+  float pos_hs, pos_ms, pos_ls;
+  double pos_scale;
 };
 
 // FP32 records: the lo part's w packs the particle's row (rz nc_y + ry, below 2^26) and, in the
@@ -195,6 +200,9 @@ struct alignas(32) D4 {
   double x, y, z, w;
 };
 
+// FP64 assignment record: idx packs the node (low 32 bits) and the input index
+__host__ __device__ inline long long rec_index(const Rec64& r) { return r.idx >> 32; }
+
 template <typename T>
 struct RecT;
 template <>
@@ -234,6 +242,8 @@ struct p3m_ctx {
   p3m::PairPoly poly{};
   dfm::PairDF* pdf = nullptr;   // FP64 path: device copy of the double-float pair-function fit
                                 // (kappa <= 6.5; otherwise nullptr and the FP64 pair function)
+  dfm::PairTab* ptab = nullptr; // FP64 path: device copy of the pair function's table
+  unsigned long long* wbound = nullptr;  // FP64 adjoint: bits of the largest |w| of a call
   int64_t n_max = 0;
   int device = 0;
   bool fp32 = false;
@@ -252,7 +262,8 @@ struct p3m_ctx {
   uint32_t* bsum = nullptr;     // scan block sums
   uint32_t* keys = nullptr;     // [n_max] key of each input particle
   uint32_t* ranks = nullptr;    // [n_max] rank within its cell
-  void* recp = nullptr;         // [n_max] sorted positions, cutoff units (2 float4 / Rec64)
+  void* recp = nullptr;         // [n_max] sorted positions, cutoff units: FP32 2 float4 each;
+                                // FP64 float4 [n_max] leading bits, then float4 [n_max] the rest
   void* recm = nullptr;         // [n_max] FP64 path: sorted assignment records (Rec64)
   void* fpp = nullptr;          // [n_max] short-range result, sorted (FP32 float4, FP64 D4)
   float4* fplo = nullptr;       // [2 n_max] FP32 path: the fine x and y parts of the
@@ -368,6 +379,10 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy);
 // into *out (FP64 contexts: nothing; their short range counts as it runs)
 void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaStream_t s);
 void launch_pp_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s);
+// the FP64 path's short range and its vector-Jacobian product (pp64.cu)
+cudaError_t pair_table_setup(p3m_ctx* c);
+void launch_pp64(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy);
+void launch_pp64_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s);
 
 // particles (particles.cu)
 void launch_bbox(const double* x, int64_t n, double* red, cudaStream_t s);

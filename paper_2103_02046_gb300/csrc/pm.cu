@@ -213,8 +213,8 @@ __device__ __forceinline__ void particle_axes(const Geom& g, const Rec64* __rest
 __device__ __forceinline__ long long orig_index(const float4* recp, uint32_t i) {
   return __float_as_int(recp[2 * i].w);  // FP32 records: hi at 2i carries the index
 }
-__device__ __forceinline__ long long orig_index(const Rec64* recp, uint32_t i) {
-  return recp[i].idx;
+__device__ __forceinline__ long long orig_index(const Rec64* recm, uint32_t i) {
+  return rec_index(recm[i]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -352,12 +352,12 @@ __device__ __forceinline__ void add128(unsigned long long* acc, long long v) {
 
 // largest sum_d |w_d| / h_d over the particles (non-negative doubles order as their bits)
 __global__ void k_dipole_bound(Geom g, const uint32_t* __restrict__ total,
-                               const Rec64* __restrict__ recp, const double* __restrict__ w,
+                               const Rec64* __restrict__ recm, const double* __restrict__ w,
                                unsigned long long* __restrict__ bound) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   double b = 0.0;
   if (i < *total) {
-    const long long idx = recp[i].idx;
+    const long long idx = rec_index(recm[i]);
     for (int d = 0; d < 3; ++d) b += fabs(w[3 * idx + d]) * g.inv_h[d];
   }
   for (int o = 16; o > 0; o >>= 1) b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
@@ -374,8 +374,7 @@ __device__ __forceinline__ double det_scale(bool dipole, const unsigned long lon
 
 template <bool kDipole>
 __global__ void k_deposit_det(Geom g, const uint32_t* __restrict__ total,
-                              const Rec64* __restrict__ recm, const Rec64* __restrict__ recp,
-                              const double* __restrict__ w,
+                              const Rec64* __restrict__ recm, const double* __restrict__ w,
                               const unsigned long long* __restrict__ bound,
                               unsigned long long* __restrict__ q128) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -386,7 +385,7 @@ __global__ void k_deposit_det(Geom g, const uint32_t* __restrict__ total,
   particle_axes(g, recm, i, A);
   double wv[3] = {0.0, 0.0, 0.0};
   if (kDipole) {
-    const long long idx = recp[i].idx;
+    const long long idx = rec_index(recm[i]);
     for (int d = 0; d < 3; ++d) wv[d] = w[3 * idx + d] * g.inv_h[d];
   }
   for (int c = 0; c < S; ++c)
@@ -939,19 +938,18 @@ void launch_deposit_det(const p3m_ctx* c, int64_t n, const double* w) {
   const size_t nn = static_cast<size_t>(c->g.n[0]) * c->g.n[1] * c->g.n[2];
   cudaMemsetAsync(c->q128, 0, 2 * sizeof(unsigned long long) * nn, c->work);
   const auto* recm = static_cast<const Rec64*>(c->recm);
-  const auto* recp = static_cast<const Rec64*>(c->recp);
   if (w) {
     cudaMemsetAsync(c->dbound, 0, sizeof(unsigned long long), c->work);
     if (n > 0)
-      k_dipole_bound<<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recp, w, c->dbound);
+      k_dipole_bound<<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm, w, c->dbound);
     if (n > 0)
-      k_deposit_det<true><<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm, recp, w,
+      k_deposit_det<true><<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm, w,
                                                                      c->dbound, c->q128);
     k_q128_to_mesh<true><<<blocks_for(nn), kThreads, 0, c->work>>>(
         c->g, c->q128, c->dbound, static_cast<double*>(c->qpad));
   } else {
     if (n > 0)
-      k_deposit_det<false><<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm, recp,
+      k_deposit_det<false><<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm,
                                                                       nullptr, c->dbound, c->q128);
     k_q128_to_mesh<false><<<blocks_for(nn), kThreads, 0, c->work>>>(
         c->g, c->q128, c->dbound, static_cast<double*>(c->qpad));
@@ -986,7 +984,7 @@ void launch_deposit(const p3m_ctx* c, int64_t n) {
         nullptr, static_cast<float*>(c->qpad));
   else
     k_deposit_tiled<double, false><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recp),
+        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recm),
         nullptr, static_cast<double*>(c->qpad));
 }
 
@@ -1004,7 +1002,7 @@ void launch_dipole_deposit(const p3m_ctx* c, int64_t n, const double* w) {
         static_cast<float*>(c->qpad));
   else
     k_deposit_tiled<double, true><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recp), w,
+        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recm), w,
         static_cast<double*>(c->qpad));
 }
 
@@ -1054,7 +1052,7 @@ void launch_vjp_gather(const p3m_ctx* c, int64_t n, int pass, const double* w, d
         c->g.ke * c->g.q * c->g.q / (c->g.rc * c->g.rc * c->g.rc));
   else
     k_vjp_gather<double><<<blocks_for(n), kThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recp),
+        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recm),
         static_cast<const double*>(c->phireal), c->n_real, w, c->acc, out, pass, nullptr, 0.0);
 }
 

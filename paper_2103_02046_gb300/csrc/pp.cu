@@ -23,26 +23,12 @@
 #include <cmath>
 #include <type_traits>
 
-#include "df_math.cuh"
-#include "p3m_internal.cuh"
+#include "pp_common.cuh"
 
 namespace p3m {
 namespace {
 
 constexpr int kThreads = 128;
-
-// Row geometry for kRows cell rows per cutoff length in y and z (Geom::rows, 1, 2 or 3): the
-// neighbour rows of a particle's row are the (2 kRows + 1)^2 rows around it, numbered y fastest;
-// the particle's own row is number `first`, and the half shell walked by the short range is
-// rows first .. last - 1 (5 of 9, 13 of 25 or 25 of 49 rows).
-template <int kRows>
-struct Rows {
-  static constexpr int reach = kRows;
-  static constexpr int span = 2 * kRows + 1;
-  static constexpr int first = span * span / 2;
-  static constexpr int last = span * span;
-  static constexpr int half = last - first;
-};
 
 // two-float accumulator (hi + lo) with Knuth's TwoSum
 struct Acc2 {
@@ -56,34 +42,6 @@ struct Acc2 {
   }
   __device__ __forceinline__ float value() const { return hi + lo; }
 };
-
-__device__ __forceinline__ void pair_terms(double r2, double kappa, double c2k, double& fco,
-                                           double& pot) {
-  const double r = sqrt(r2);
-  const double x = kappa * r;
-  const double ec = erfc(x);
-  const double ex = exp(-x * x);
-  pot = ec / r;
-  fco = (pot + c2k * ex) / r2;
-}
-
-template <int kBlk = kThreads>
-__device__ __forceinline__ void block_reduce_add(double v, double* dst) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __shared__ double ws[kBlk / 32];
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double s = threadIdx.x < kBlk / 32 ? ws[threadIdx.x] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) atomicAdd(dst, s);
-  }
-}
-
-__device__ __forceinline__ void warp_add_u64(unsigned long long v, unsigned long long* dst) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
-}
 
 // Calls visit(j0, j1) for every neighbour row of the query point (px, py, pz) (cutoff units)
 // that can hold particles within distance 1, with [j0, j1) the sorted range of its cells whose
@@ -118,13 +76,6 @@ __device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restri
     }
   }
 }
-
-// ------------------------------------------------------------------------------------------
-// Position access for the FP64 adjoint kernel.
-// ------------------------------------------------------------------------------------------
-struct PosD {
-  const Rec64* __restrict__ r;
-};
 
 // ------------------------------------------------------------------------------------------
 // FP32 short range: each unordered pair once (Newton's third law), each lane holding two
@@ -313,34 +264,6 @@ __device__ __forceinline__ void pair_poly(const PairPoly& P, float r2, float& fc
   const float ex = exp2f(-P.kappa2_log2e * r2);
   pot = R * ex * rinv;
   fco = fmaf(P.c2k, ex, pot) * (rinv * rinv);
-}
-
-// Sorted range [j0, j1) of neighbour row r (y fastest, Rows::first = the particle's own row
-// (cy, cz)) that can hold particles within distance 1 of (px, py, pz); empty if none can. The
-// rectangle distance and the x half-width carry the search slack, as in for_rows.
-template <int kRows>
-__device__ __forceinline__ void row_range(const Geom& g, const uint32_t* __restrict__ starts,
-                                          float px, float py, float pz, int cy, int cz, int r,
-                                          uint32_t& j0, uint32_t& j1) {
-  using R = Rows<kRows>;
-  j0 = j1 = 0;
-  const int ry = cy + (r % R::span) - R::reach, rz = cz + (r / R::span) - R::reach;
-  if (ry < 0 || ry >= g.nc[1] || rz < 0 || rz >= g.nc[2]) return;
-  const float slack = g.slack_f;
-  const float cwy = g.cw_f[1], cwz = g.cw_f[2];
-  const float yl = ry * cwy, yh = yl + cwy, zl = rz * cwz, zh = zl + cwz;
-  const float dy = fmaxf((py < yl ? yl - py : (py > yh ? py - yh : 0.f)) - slack, 0.f);
-  const float dz = fmaxf((pz < zl ? zl - pz : (pz > zh ? pz - zh : 0.f)) - slack, 0.f);
-  const float d2 = dy * dy + dz * dz;
-  if (d2 >= 1.f) return;
-  const float w = sqrtf(1.f - d2) + slack;
-  const float iwx = g.inv_cw_f[0];
-  const int c0 = max(static_cast<int>(floorf((px - w) * iwx)), 0);
-  const int c1 = min(static_cast<int>(floorf((px + w) * iwx)), g.nc[0] - 1);
-  if (c0 > c1) return;
-  const uint32_t base = (static_cast<uint32_t>(rz) * g.nc[1] + ry) * g.nc[0];
-  j0 = starts[base + c0];
-  j1 = starts[base + c1 + 1];
 }
 
 // b's own runs (particle ib in row row_b), for a lane whose two particles sit in different rows
@@ -913,324 +836,16 @@ __global__ void k_gather_w(const uint32_t* __restrict__ total, const float4* __r
                       static_cast<float>(w[3 * idx + 2]), 0.f);
 }
 
-// ------------------------------------------------------------------------------------------
-// FP64 short range: each unordered pair once, as in the FP32 kernel: particle i takes the pairs
-// with j > i in sorted order (every one of the 25 neighbour rows is clipped to j > i, so this
-// holds however the row of i was rounded) and adds the reaction to j with FP64 reductions into
-// the zeroed result. Rows are walked in lockstep. FP64 arithmetic is scarce on this part, so the
-// walk itself runs in FP32: the row search and a distance prefilter on the leading 24 bits of
-// each coordinate (within the search slack of the exact test). Candidates that pass wait in a
-// per-lane ring in shared memory and are evaluated, a batch of one per lane, whenever some lane's
-// ring is full: the exact FP64 separation decides the pair (r^2 < 1 in FP64, as the definition
-// reads), and the pair terms follow (in double-float, or FP64 for large kappa), with most lanes
-// busy.
-// ------------------------------------------------------------------------------------------
-constexpr int kRingJ = 16;  // queued candidates per lane of the FP64 short range
-
-// The FP64 path's pair function in double-float arithmetic (df_math.cuh): the fit table copied
-// into shared memory by the block (only the intervals and degrees in use), s = rho^2 split into
-// two floats with integer operations, the results widened exactly and summed in FP64.
-struct DFTable {
-  dfm::PairConsts k;
-  dfm::Coef coef[dfm::kMaxIntervals];
-};
-
-__device__ __forceinline__ void load_df_table(const dfm::PairDF* __restrict__ src, DFTable& dst) {
-  constexpr int kWords = sizeof(dfm::PairConsts) / sizeof(uint32_t);
-  static_assert(sizeof(dfm::PairConsts) % sizeof(uint32_t) == 0, "copied in words");
-  const uint32_t* s = reinterpret_cast<const uint32_t*>(&src->k);
-  uint32_t* d = reinterpret_cast<uint32_t*>(&dst.k);
-  for (int t = threadIdx.x; t < kWords; t += blockDim.x) d[t] = s[t];
-  const int nint = src->k.nint, deg1 = src->k.deg + 1;
-  for (int t = threadIdx.x; t < nint * deg1; t += blockDim.x)
-    dst.coef[t / deg1][t % deg1] = src->coef[t / deg1][t % deg1];
-  __syncthreads();
-}
-
-__device__ __forceinline__ double df_to_double(dfm::F2 v) {
-  return float_to_double_exact(v.hi) + float_to_double_exact(v.lo);
-}
-
-__device__ __forceinline__ void pair_terms_df(const DFTable& T, double r2, double& fco,
-                                              double& pot) {
-  const DF sd = df_from_double(r2);
-  const dfm::PairOut o = dfm::pair_df(T.k, T.coef, dfm::F2{sd.hi, sd.lo});
-  fco = df_to_double(o.fco);
-  pot = df_to_double(o.pot);
-}
-
-// the force coefficient alone (no potential: the energy is not asked for)
-__device__ __forceinline__ double pair_fco_df(const DFTable& T, double r2) {
-  const DF sd = df_from_double(r2);
-  return df_to_double(dfm::pair_df(T.k, T.coef, dfm::F2{sd.hi, sd.lo}).fco);
-}
-
-__device__ __forceinline__ void pair_hess_dfd(const DFTable& T, double r2, double& fco,
-                                              double& dfr) {
-  const DF sd = df_from_double(r2);
-  dfm::F2 f, d;
-  dfm::pair_hess_df(T.k, T.coef, dfm::F2{sd.hi, sd.lo}, f, d);
-  fco = df_to_double(f);
-  dfr = df_to_double(d);
-}
-
-template <int kRows>
-__device__ __forceinline__ void row_range64(const Geom& g, const uint32_t* __restrict__ starts,
-                                            double px, double py, double pz, int cy, int cz,
-                                            int r, uint32_t& j0, uint32_t& j1) {
-  using R = Rows<kRows>;
-  j0 = j1 = 0;
-  const int ry = cy + (r % R::span) - R::reach, rz = cz + (r / R::span) - R::reach;
-  if (ry < 0 || ry >= g.nc[1] || rz < 0 || rz >= g.nc[2]) return;
-  const double slack = g.slack;
-  const double yl = ry * g.cw[1], yh = yl + g.cw[1], zl = rz * g.cw[2], zh = zl + g.cw[2];
-  const double dy = fmax((py < yl ? yl - py : (py > yh ? py - yh : 0.0)) - slack, 0.0);
-  const double dz = fmax((pz < zl ? zl - pz : (pz > zh ? pz - zh : 0.0)) - slack, 0.0);
-  const double d2 = dy * dy + dz * dz;
-  if (d2 >= 1.0) return;
-  const double w = sqrt(1.0 - d2) + slack;
-  const int c0 = max(static_cast<int>(floor((px - w) * g.inv_cw[0])), 0);
-  const int c1 = min(static_cast<int>(floor((px + w) * g.inv_cw[0])), g.nc[0] - 1);
-  if (c0 > c1) return;
-  const uint32_t base = (static_cast<uint32_t>(rz) * g.nc[1] + ry) * g.nc[0];
-  j0 = starts[base + c0];
-  j1 = starts[base + c1 + 1];
-}
-
-// kDet (deterministic = 1): every ordered pair is evaluated by its own particle (all rows of the
-// block, j != i), with no reductions: each particle's sum runs in the fixed sorted order and is
-// stored as is, together with its potential (w), from which the energy is summed in a fixed
-// order afterwards.
-template <int kRows, bool kDet, bool kDF, bool kPot>
-__global__ void __launch_bounds__(kThreads)
-    k_pp_f64(Geom g, const uint32_t* __restrict__ total, const Rec64* __restrict__ rec,
-             const Rec64* __restrict__ recm, const uint32_t* __restrict__ starts,
-             D4* __restrict__ fpp, double* __restrict__ energy,
-             unsigned long long* __restrict__ pairs, const dfm::PairDF* __restrict__ dftab) {
-  __shared__ typename std::conditional<kDF, DFTable, char>::type dft_s[1];
-  if constexpr (kDF) load_df_table(dftab, dft_s[0]);
-  __shared__ uint32_t ringj_s[kThreads / 32][kRingJ][32];
-  uint32_t(*ringj)[32] = ringj_s[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const uint32_t N = *total;
-  const uint32_t i = blockIdx.x * kThreads + threadIdx.x;
-  const bool alive = i < N;
-  const double kappa = g.kappa_eff;
-  const double c2k = 2.0 * g.kappa_eff * 0.56418958354775628695;
-  // lanes past the last particle compare record 0 with itself (separation 0, never a pair)
-  const uint32_t ie = alive ? i : 0u;
-  const Rec64 me = rec[ie];
-  const double px = me.u[0], py = me.u[1], pz = me.u[2];
-  // FP32 copies (the leading 24 bits) for the search and the distance prefilter; the search
-  // slack exceeds their truncation error (2^-23 of the coordinate, twice, on each axis)
-  const float pxf = df_from_double(px).hi, pyf = df_from_double(py).hi,
-              pzf = df_from_double(pz).hi;
-  const float thr = (1.f + g.slack_f) * (1.f + g.slack_f);
-  // the row the sort put the particle in (two particles closer than r_c sit in sort rows at most
-  // kRows apart, whatever the rounding of either binning)
-  const uint32_t row = static_cast<uint32_t>(static_cast<unsigned long long>(recm[ie].idx) >> 32);
-  const int cy = static_cast<int>(row % static_cast<uint32_t>(g.nc[1]));
-  const int cz = static_cast<int>(row / static_cast<uint32_t>(g.nc[1]));
-  double sum[4] = {0.0, 0.0, 0.0, 0.0};
-  unsigned int np = 0, ncand = 0;  // pairs found, records tested
-  int head = 0, cnt = 0;
-  // one queued candidate per lane: the exact FP64 separation decides, then the pair terms
-  auto evaluate = [&]() {
-    const bool has = cnt > 0;
-    const uint32_t j = has ? ringj[head & (kRingJ - 1)][lane] : ie;
-    const Rec64 rj = rec[j];
-    const double rx = px - rj.u[0], ry = py - rj.u[1], rz = pz - rj.u[2];
-    const double r2 = rx * rx + ry * ry + rz * rz;
-    const bool hit = has && r2 < 1.0 && r2 > 0.0;
-    double fco, pot = 0.0;
-    if constexpr (kDF) {
-      if constexpr (kPot)
-        pair_terms_df(dft_s[0], hit ? r2 : 0.5, fco, pot);
-      else
-        fco = pair_fco_df(dft_s[0], hit ? r2 : 0.5);
-    } else {
-      pair_terms(hit ? r2 : 0.5, kappa, c2k, fco, pot);
-    }
-    if (hit) {
-      // the reaction's components, -fco (xi_i - xi_j): the own sum subtracts them
-      const double nf = -fco;
-      const double gx = nf * rx, gy = nf * ry, gz = nf * rz;
-      sum[0] -= gx;
-      sum[1] -= gy;
-      sum[2] -= gz;
-      if constexpr (kPot) sum[3] += pot;
-      ++np;
-      if (!kDet) {
-        double* fj = &fpp[j].x;
-        // the potential is summed on the owner's side only: j's fourth component stays unused
-        atomicAdd(fj, gx);
-        atomicAdd(fj + 1, gy);
-        atomicAdd(fj + 2, gz);
-      }
-    }
-    head += has;
-    cnt -= has;
-  };
-  for (int r = 0; r < Rows<kRows>::last; ++r) {
-    uint32_t j0 = 0, j1 = 0;
-    if (alive) {
-      row_range<kRows>(g, starts, pxf, pyf, pzf, cy, cz, r, j0, j1);
-      if (!kDet) j0 = max(j0, i + 1);
-      j1 = max(j1, j0);
-    }
-    const int len = static_cast<int>(j1 - j0);
-    ncand += static_cast<unsigned>(len);
-    int maxlen = len;
-    for (int o = 16; o > 0; o >>= 1) maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
-    for (int t = 0; t < maxlen; ++t) {
-      const bool v = t < len;
-      const uint32_t j = v ? j0 + t : ie;
-      const Rec64 rj = rec[j];
-      const float dx = pxf - df_from_double(rj.u[0]).hi;
-      const float dy = pyf - df_from_double(rj.u[1]).hi;
-      const float dz = pzf - df_from_double(rj.u[2]).hi;
-      if (alive && v && j != i && fmaf(dx, dx, fmaf(dy, dy, dz * dz)) < thr) {
-        ringj[(head + cnt) & (kRingJ - 1)][lane] = j;
-        ++cnt;
-      }
-      if (__any_sync(0xffffffffu, cnt == kRingJ)) evaluate();
-    }
-  }
-  while (__any_sync(0xffffffffu, cnt > 0)) evaluate();
-  const double pair_pot = sum[3];
-  unsigned long long ni = 0;
-  if (alive && g.pp_bc && pz - 0.5 * g.img_c < 1.0) {
-    // images within r_c of particles less than r_c above the cathode (rare): plain loop
-    for_rows<double>(g, starts, px, py, g.img_c - pz, [&](uint32_t ja, uint32_t jb) {
-      for (uint32_t jj = ja; jj < jb; ++jj) {
-        const Rec64 rj = rec[jj];
-        const double ax = px - rj.u[0], ay = py - rj.u[1], az = pz + rj.u[2] - g.img_c;
-        const double r2 = ax * ax + ay * ay + az * az;
-        if (r2 < 1.0 && r2 > 0.0) {
-          double fco, pot;
-          if constexpr (kDF)
-            pair_terms_df(dft_s[0], r2, fco, pot);
-          else
-            pair_terms(r2, kappa, c2k, fco, pot);
-          sum[0] -= fco * ax;
-          sum[1] -= fco * ay;
-          sum[2] -= fco * az;
-          if constexpr (kPot) sum[3] -= pot;
-          ++ni;
-        }
-      }
-    });
-  }
-  if (kDet) {
-    // sum_i phi_i is formed from w in a fixed order by the caller
-    if (alive) fpp[i] = D4{sum[0], sum[1], sum[2], sum[3]};
-  } else {
-    if (alive) {
-      double* fi = &fpp[i].x;
-      for (int c = 0; c < 3; ++c) atomicAdd(fi + c, sum[c]);  // the potential: energy only
-    }
-    // sum_i phi_i over ordered pairs: each pair's potential was taken once here, plus images
-    if (energy) block_reduce_add(alive ? sum[3] + pair_pot : 0.0, energy);
-  }
-  warp_add_u64(kDet ? np : 2ull * np, pairs);
-  warp_add_u64(ni, pairs + 1);
-  warp_add_u64(ncand, pairs + 2);
-}
-
-// Vector-Jacobian product of the short-range force map, into acc (sorted order):
-//   free pairs:  acc_i += H(d_ij) (w_i - w_j)
-//   image pairs: acc_i -= H(d_ij) (w_i - S w_j)   (S = diag(1, 1, -1), image charge -q)
-// H(d) = [phi(rho) I + (phi'(rho)/rho) d d^T] (times k_e q^2 / r_c^3). The force map is the
-// gradient of an energy, so its Jacobian is symmetric and this gather equals J^T w.
-template <typename T>
-__device__ __forceinline__ void pair_hess(T r2, T kappa, T c2k, T& fco, T& dfr) {
-  const T r = sqrt(r2);
-  const T x = kappa * r;
-  const T ex = exp(-x * x);
-  const T ec = erfc(x);
-  const T A = ec / r + c2k * ex;
-  const T dA = -c2k * ex / r - ec / r2 - T(2) * kappa * kappa * r * c2k * ex;
-  fco = A / r2;
-  dfr = (dA / r2 - T(2) * A / (r2 * r)) / r;
-}
-
-// FP64 vector-Jacobian product of the short-range force map (every ordered pair, one thread
-// per particle): acc_i = scale sum_j H(d_ij) (w_i - w_j) - scale sum_j H(d_ij') (w_i - S w_j)
-// over image pairs (pp_bc).
-template <bool kDF>
-__global__ void __launch_bounds__(kThreads)
-    k_pp_vjp(Geom g, const uint32_t* __restrict__ total, PosD pos,
-             const uint32_t* __restrict__ starts, const double* __restrict__ w,
-             double* __restrict__ acc, double scale, const dfm::PairDF* __restrict__ dftab) {
-  __shared__ typename std::conditional<kDF, DFTable, char>::type dft_s[1];
-  if constexpr (kDF) load_df_table(dftab, dft_s[0]);
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= *total) return;
-  auto hess = [&](double r2, double& fco, double& dfr) {
-    if constexpr (kDF)
-      pair_hess_dfd(dft_s[0], r2, fco, dfr);
-    else
-      pair_hess(r2, g.kappa_eff, 2.0 * g.kappa_eff * 0.56418958354775628695, fco, dfr);
-  };
-  const double kappa = g.kappa_eff;
-  const double c2k = 2.0 * g.kappa_eff * 0.56418958354775628695;
-  const Rec64 me = pos.r[i];
-  const double pi[3] = {me.u[0], me.u[1], me.u[2]};
-  const long long idx = me.idx;
-  const double wi[3] = {w[3 * idx], w[3 * idx + 1], w[3 * idx + 2]};
-  double out[3] = {0.0, 0.0, 0.0};
-  for_rows<double>(g, starts, pi[0], pi[1], pi[2], [&](uint32_t j0, uint32_t j1) {
-    for (uint32_t j = j0; j < j1; ++j) {
-      if (j == i) continue;
-      const Rec64 rj = pos.r[j];
-      const double rx = pi[0] - rj.u[0], ry = pi[1] - rj.u[1], rz = pi[2] - rj.u[2];
-      const double r2 = rx * rx + ry * ry + rz * rz;
-      if (r2 < 1.0 && r2 > 0.0) {
-        double fco, dfr;
-        hess(r2, fco, dfr);
-        const double v0 = wi[0] - w[3 * rj.idx];
-        const double v1 = wi[1] - w[3 * rj.idx + 1];
-        const double v2 = wi[2] - w[3 * rj.idx + 2];
-        const double dv = rx * v0 + ry * v1 + rz * v2;
-        out[0] += fco * v0 + dfr * dv * rx;
-        out[1] += fco * v1 + dfr * dv * ry;
-        out[2] += fco * v2 + dfr * dv * rz;
-      }
-    }
-  });
-  if (g.pp_bc && pi[2] - 0.5 * g.img_c < 1.0) {
-    for_rows<double>(g, starts, pi[0], pi[1], g.img_c - pi[2], [&](uint32_t j0, uint32_t j1) {
-      for (uint32_t j = j0; j < j1; ++j) {
-        const Rec64 rj = pos.r[j];
-        const double rx = pi[0] - rj.u[0], ry = pi[1] - rj.u[1];
-        const double rz = pi[2] + rj.u[2] - g.img_c;
-        const double r2 = rx * rx + ry * ry + rz * rz;
-        if (r2 < 1.0 && r2 > 0.0) {
-          double fco, dfr;
-          hess(r2, fco, dfr);
-          const double v0 = wi[0] - w[3 * rj.idx];
-          const double v1 = wi[1] - w[3 * rj.idx + 1];
-          const double v2 = wi[2] + w[3 * rj.idx + 2];  // w_i - S w_j
-          const double dv = rx * v0 + ry * v1 + rz * v2;
-          out[0] -= fco * v0 + dfr * dv * rx;
-          out[1] -= fco * v1 + dfr * dv * ry;
-          out[2] -= fco * v2 + dfr * dv * rz;
-        }
-      }
-    });
-  }
-  acc[3 * i] = scale * out[0];
-  acc[3 * i + 1] = scale * out[1];
-  acc[3 * i + 2] = scale * out[2];
-}
-
 }  // namespace
 
 void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
   if (n == 0) return;
-  const unsigned blocks = static_cast<unsigned>((n + kThreads - 1) / kThreads);
+  if (!c->fp32) {
+    launch_pp64(c, n, s, want_energy);
+    return;
+  }
   const uint32_t* total = c->starts + c->nkeys;
-  if (c->fp32) {
+  {
     // the kernel adds each pair's force to both particles: the result (coarse, fine and big
     // parts) starts at zero
     float4* fbig = c->fplo + c->n_max;
@@ -1269,35 +884,6 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
       case 14: run(k_pp_f32<14, 1>, k_pp_f32<14, 2>, k_pp_f32<14, 3>); break;
       default: run(k_pp_f32<15, 1>, k_pp_f32<15, 2>, k_pp_f32<15, 3>); break;
     }
-  } else {
-    auto pick = [&](auto k1, auto k2, auto k3) {
-      return c->g.rows == 1 ? k1 : (c->g.rows == 2 ? k2 : k3);
-    };
-    // the pair potentials are summed for the energy or the deterministic mode's fixed-order sum
-    const bool pot = c->det || want_energy;
-    auto kern = c->pdf
-                    ? (c->det ? pick(k_pp_f64<1, true, true, true>, k_pp_f64<2, true, true, true>,
-                                     k_pp_f64<3, true, true, true>)
-                              : (pot ? pick(k_pp_f64<1, false, true, true>,
-                                            k_pp_f64<2, false, true, true>,
-                                            k_pp_f64<3, false, true, true>)
-                                     : pick(k_pp_f64<1, false, true, false>,
-                                            k_pp_f64<2, false, true, false>,
-                                            k_pp_f64<3, false, true, false>)))
-                    : (c->det ? pick(k_pp_f64<1, true, false, true>, k_pp_f64<2, true, false, true>,
-                                     k_pp_f64<3, true, false, true>)
-                              : (pot ? pick(k_pp_f64<1, false, false, true>,
-                                            k_pp_f64<2, false, false, true>,
-                                            k_pp_f64<3, false, false, true>)
-                                     : pick(k_pp_f64<1, false, false, false>,
-                                            k_pp_f64<2, false, false, false>,
-                                            k_pp_f64<3, false, false, false>)));
-    if (!c->det) cudaMemsetAsync(c->fpp, 0, sizeof(D4) * static_cast<size_t>(n), s);
-    kern<<<blocks, kThreads, 0, s>>>(c->g, total, static_cast<const Rec64*>(c->recp),
-                                     static_cast<const Rec64*>(c->recm), c->starts,
-                                     static_cast<D4*>(c->fpp), pot ? c->energy_acc : nullptr,
-                                     c->pair_acc, c->pdf);
-    if (c->det) launch_det_sum_pp(c, n, s);
   }
 }
 
@@ -1315,9 +901,13 @@ void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaS
 
 void launch_pp_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s) {
   if (n == 0) return;
+  if (!c->fp32) {
+    launch_pp64_vjp(c, n, w, s);
+    return;
+  }
   const unsigned blocks = static_cast<unsigned>((n + kThreads - 1) / kThreads);
   const uint32_t* total = c->starts + c->nkeys;
-  if (c->fp32) {
+  {
     // weights in sorted order (in acc, free until the mesh gather), result in fpp (cutoff
     // units; the mesh gather scales it)
     float4* ws = reinterpret_cast<float4*>(c->acc);
@@ -1346,12 +936,6 @@ void launch_pp_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s)
       case 14: run(k_pp_vjp_f32<14, 1>, k_pp_vjp_f32<14, 2>, k_pp_vjp_f32<14, 3>); break;
       default: run(k_pp_vjp_f32<15, 1>, k_pp_vjp_f32<15, 2>, k_pp_vjp_f32<15, 3>); break;
     }
-  } else {
-    // d/dxi of (k_e q^2 / r_c^2) f(rho): one more factor 1/r_c
-    const double scale = c->g.ke * c->g.q * c->g.q / (c->g.rc * c->g.rc * c->g.rc);
-    auto kern = c->pdf ? k_pp_vjp<true> : k_pp_vjp<false>;
-    kern<<<blocks, kThreads, 0, s>>>(c->g, total, PosD{static_cast<const Rec64*>(c->recp)},
-                                     c->starts, w, c->acc, scale, c->pdf);
   }
 }
 

@@ -184,14 +184,14 @@ template <bool kFP32>
 __global__ void k_scatter(Geom g, const double* __restrict__ x, int64_t n,
                           uint32_t* __restrict__ keys, const uint32_t* __restrict__ ranks,
                           const uint32_t* __restrict__ starts, void* __restrict__ recp,
-                          void* __restrict__ recm) {
+                          void* __restrict__ recm, int64_t n_max) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
   const uint32_t key = keys[i];
   if (key == kInvalidKey) return;
   const uint32_t pos = starts[key] + ranks[i];
   keys[i] = pos;  // from here on keys[i] is the sorted position of input particle i
-  if (kFP32) {
+  if constexpr (kFP32) {
     // FP32 record (one 32-byte sector): the position in cutoff units as hi + lo from
     // double-float arithmetic (about 2^-46 relative), the input index, the row, and per axis
     // the node correction. The mesh kernels recompute the assignment node from hi + lo
@@ -221,45 +221,49 @@ __global__ void k_scatter(Geom g, const double* __restrict__ x, int64_t n,
     float4* r = reinterpret_cast<float4*>(recp) + 2 * static_cast<size_t>(pos);
     r[0] = make_float4(hi[0], hi[1], hi[2], __int_as_float(static_cast<int>(i)));
     r[1] = make_float4(lo[0], lo[1], lo[2], __uint_as_float(row | (code << kRowBits)));
-    return;
-  }
-  double xr[3], u[3];
-  int c[3];
-  for (int d = 0; d < 3; ++d) {
-    const double v = x[3 * i + d];
-    const double dv = v - g.lo[d];
-    xr[d] = dv * g.inv_rc;
-    // node from an FP32 estimate unless it is within 1e-3 of a knot; then from the exact s
-    const float sf = static_cast<float>(dv) * g.inv_h_f[d];
-    const float cf = (g.order == 2) ? floorf(sf + 0.5f) : floorf(sf);
-    const float kl = (g.order == 2) ? cf - 0.5f : cf;
-    double cn;
-    if (fabsf(sf - kl) < 1e-3f || fabsf(sf - kl - 1.f) < 1e-3f) {
-      const double s = mesh_coord(g, v, d);
-      cn = (g.order == 2) ? floor(s + 0.5) : floor(s);
-      u[d] = s - cn;
-    } else {
-      cn = static_cast<double>(cf);
-      u[d] = fma(-cn, g.h[d], dv) * g.inv_h[d];
+  } else {
+    unsigned long long xq[3];
+    double u[3];
+    int c[3];
+    for (int d = 0; d < 3; ++d) {
+      const double v = x[3 * i + d];
+      const double dv = v - g.lo[d];
+      xq[d] = __double2ull_rn(fmax(dv * g.inv_rc, 0.0) * g.pos_scale);
+      // node from an FP32 estimate unless it is within 1e-3 of a knot; then from the exact s
+      const float sf = static_cast<float>(dv) * g.inv_h_f[d];
+      const float cf = (g.order == 2) ? floorf(sf + 0.5f) : floorf(sf);
+      const float kl = (g.order == 2) ? cf - 0.5f : cf;
+      double cn;
+      if (fabsf(sf - kl) < 1e-3f || fabsf(sf - kl - 1.f) < 1e-3f) {
+        const double s = mesh_coord(g, v, d);
+        cn = (g.order == 2) ? floor(s + 0.5) : floor(s);
+        u[d] = s - cn;
+      } else {
+        cn = static_cast<double>(cf);
+        u[d] = fma(-cn, g.h[d], dv) * g.inv_h[d];
+      }
+      c[d] = static_cast<int>(cn);
     }
-    c[d] = static_cast<int>(cn);
-  }
-  const uint32_t node = pack_node(c[0], c[1], c[2]);
-  {
-    Rec64 r;
-    r.u[0] = xr[0];
-    r.u[1] = xr[1];
-    r.u[2] = xr[2];
-    r.idx = static_cast<long long>(i);
-    reinterpret_cast<Rec64*>(recp)[pos] = r;
+    const uint32_t node = pack_node(c[0], c[1], c[2]);
+    // position: 24 + 24 + 8 bits of the fixed-point value per axis, each piece exact in FP32; the
+    // cell row with the leading pieces, which the short range centres its row block on (the row
+    // the sort used, so that the search slack argument holds)
+    const uint32_t row = key / static_cast<uint32_t>(g.nc[0]);
+    float h[3], q[3];
+    uint32_t low = 0;
+    for (int d = 0; d < 3; ++d) {
+      h[d] = static_cast<float>(static_cast<uint32_t>(xq[d] >> 32)) * g.pos_hs;
+      q[d] = static_cast<float>(static_cast<uint32_t>(xq[d] >> 8) & 0xffffffu) * g.pos_ms;
+      low |= (static_cast<uint32_t>(xq[d]) & 0xffu) << (8 * d);
+    }
+    float4* r = reinterpret_cast<float4*>(recp);
+    r[pos] = make_float4(h[0], h[1], h[2], __uint_as_float(row));
+    r[n_max + pos] = make_float4(q[0], q[1], q[2], __uint_as_float(low));
     Rec64 m;
     m.u[0] = u[0];
     m.u[1] = u[1];
     m.u[2] = u[2];
-    // the node in the low 32 bits; above it the particle's cell row, which the FP64 short range
-    // centres its row block on (the row the sort used, so that the search slack argument holds)
-    m.idx = static_cast<long long>(node) |
-            (static_cast<long long>(key / static_cast<uint32_t>(g.nc[0])) << 32);
+    m.idx = static_cast<long long>(node) | (static_cast<long long>(i) << 32);
     reinterpret_cast<Rec64*>(recm)[pos] = m;
   }
 }
@@ -269,24 +273,27 @@ __global__ void k_scatter(Geom g, const double* __restrict__ x, int64_t n,
 // re-orders its records by input index (insertion sort; cells hold a few particles) and updates
 // the sorted position kept in keys. Every later sum then runs in an order fixed by the input.
 __global__ void k_cell_order(uint64_t nkeys, const uint32_t* __restrict__ starts,
-                             Rec64* __restrict__ recp, Rec64* __restrict__ recm,
-                             uint32_t* __restrict__ keys) {
+                             float4* __restrict__ ph, float4* __restrict__ pml,
+                             Rec64* __restrict__ recm, uint32_t* __restrict__ keys) {
   const uint64_t c = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
   if (c >= nkeys) return;
   const uint32_t j0 = starts[c], j1 = starts[c + 1];
   if (j1 - j0 < 2) return;
   for (uint32_t j = j0 + 1; j < j1; ++j) {
-    const Rec64 p = recp[j], m = recm[j];
+    const float4 h = ph[j], q = pml[j];
+    const Rec64 m = recm[j];
     uint32_t k = j;
-    while (k > j0 && recp[k - 1].idx > p.idx) {
-      recp[k] = recp[k - 1];
+    while (k > j0 && rec_index(recm[k - 1]) > rec_index(m)) {
+      ph[k] = ph[k - 1];
+      pml[k] = pml[k - 1];
       recm[k] = recm[k - 1];
       --k;
     }
-    recp[k] = p;
+    ph[k] = h;
+    pml[k] = q;
     recm[k] = m;
   }
-  for (uint32_t j = j0; j < j1; ++j) keys[recp[j].idx] = j;
+  for (uint32_t j = j0; j < j1; ++j) keys[rec_index(recm[j])] = j;
 }
 
 inline unsigned grid_for(int64_t n, int threads) {
@@ -316,13 +323,14 @@ void launch_scatter(const p3m_ctx* c, const double* x, int64_t n) {
   if (n == 0) return;
   if (c->fp32)
     k_scatter<true><<<grid_for(n, kBinThreads), kBinThreads, 0, c->work>>>(
-        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm);
+        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max);
   else {
     k_scatter<false><<<grid_for(n, kBinThreads), kBinThreads, 0, c->work>>>(
-        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm);
+        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max);
     if (c->det)
       k_cell_order<<<static_cast<unsigned>((c->nkeys + kBinThreads - 1) / kBinThreads),
-                     kBinThreads, 0, c->work>>>(c->nkeys, c->starts, static_cast<Rec64*>(c->recp),
+                     kBinThreads, 0, c->work>>>(c->nkeys, c->starts, static_cast<float4*>(c->recp),
+                                                static_cast<float4*>(c->recp) + c->n_max,
                                                 static_cast<Rec64*>(c->recm), c->keys);
   }
 }

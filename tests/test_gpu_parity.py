@@ -784,3 +784,23 @@ def test_workload_gradient_4096_200_steps():
     # measured 6e-15 (x0) and 3e-16 (p0)
     assert rel(gx0, ogx) <= 1e-10
     assert rel(gp0, ogp) <= 1e-10
+
+
+@pytest.mark.parametrize("n", [1, 31, 9727, 9728, 19457, 38911, 38912])
+@pytest.mark.parametrize("rows", [1, 3])
+def test_fp64_lane_groups(n, rows):
+    # FP64 short range: the lanes that share a particle (32, 16, 8 or 4, by the particle count)
+    # give the same pairs and forces on both sides of every change, for cell rows as wide as the
+    # cutoff and a third of it, with image pairs
+    x = np.random.default_rng(n).uniform(-1e-3, 1e-3, size=(n, 3))
+    x[:, 2] += 1.02e-3
+    box = np.array([[-1e-3, -1e-3, 0.0], [1e-3, 1e-3, 2.04e-3]])
+    P = O.auto_mesh(box, 24, rc_over_h=1.5, pm_bc=1, pp_bc=1, z_cathode=0.0)
+    ref = O.forces(x, P)
+    ctx = p3m().Context(gpu_params(P, 0, search_rows=rows, search_xcells=4), n)
+    f = ctx.forces(cuda(x))
+    pairs = ctx.pair_count()
+    ctx.sync()
+    assert pairs == (ref.pairs, ref.image_pairs)
+    assert rel(f, ref.F) <= TOL[0]
+    ctx.close()
