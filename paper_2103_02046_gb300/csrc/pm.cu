@@ -229,6 +229,17 @@ constexpr int kDepItems = 4;
 constexpr int kDepPerBlock = kDepThreads * kDepItems;
 constexpr int kTileBytes = 32768;
 
+// The charged block n^3 of the doubled mesh to zero (grid: x-y plane by z plane). As one kernel: a
+// pitched 3D memset of the same block takes 200 us and more, whatever the mesh (measured: the
+// deposit stage of 261,121 particles on 64^3 284 us with it, 40 us with this).
+template <typename T>
+__global__ void k_zero_block(Geom g, T* __restrict__ q) {
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= static_cast<uint32_t>(g.n[0]) * static_cast<uint32_t>(g.n[1])) return;
+  const uint32_t y = t / static_cast<uint32_t>(g.n[0]), x = t - y * g.n[0];
+  q[real_index(g, x, y, blockIdx.y)] = T(0);
+}
+
 template <typename T, bool kDipole>
 __global__ void __launch_bounds__(kDepThreads)
     k_deposit_tiled(Geom g, const uint32_t* __restrict__ total,
@@ -928,9 +939,12 @@ cudaError_t build_green(p3m_ctx* c) {
 }
 
 void launch_zero_block(const p3m_ctx* c) {
-  const size_t es = c->fp32 ? sizeof(float) : sizeof(double);
-  cudaPitchedPtr pp = make_cudaPitchedPtr(c->qpad, es * c->g.M[0], es * c->g.M[0], c->g.M[1]);
-  cudaMemset3DAsync(pp, 0, make_cudaExtent(es * c->g.n[0], c->g.n[1], c->g.n[2]), c->work);
+  const Geom& g = c->g;
+  const dim3 grid(blocks_for(static_cast<uint64_t>(g.n[0]) * g.n[1]), g.n[2]);
+  if (c->fp32)
+    k_zero_block<float><<<grid, kThreads, 0, c->work>>>(g, static_cast<float*>(c->qpad));
+  else
+    k_zero_block<double><<<grid, kThreads, 0, c->work>>>(g, static_cast<double*>(c->qpad));
 }
 
 void launch_deposit_det(const p3m_ctx* c, int64_t n, const double* w) {
