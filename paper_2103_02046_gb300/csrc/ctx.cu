@@ -340,10 +340,12 @@ p3m_status check_n(p3m_ctx* c, int64_t n) {
   return P3M_OK;
 }
 
-void sort_particles(p3m_ctx* c, const double* x, int64_t n, double* f_zero) {
+// evaluation: a force evaluation follows (its accumulators start at zero); pp: and its short range
+void sort_particles(p3m_ctx* c, const double* x, int64_t n, double* f_zero, bool evaluation,
+                    bool pp) {
   launch_bin(c, x, n, f_zero);
-  launch_scan(c);
-  launch_scatter(c, x, n);
+  launch_scan(c, evaluation);
+  launch_scatter(c, x, n, pp);
   c->last_n = n;
 }
 
@@ -447,10 +449,8 @@ p3m_status mesh_solve(p3m_ctx* c, bool want_phi, bool want_diff, bool want_energ
 p3m_status forces_impl(p3m_ctx* c, const double* x, int64_t n, double* f, double* energy,
                        int parts) {
   cudaStream_t st = c->work;
-  cudaMemsetAsync(c->energy_acc, 0, 2 * sizeof(double), st);
-  cudaMemsetAsync(c->pair_acc, 0, 3 * sizeof(unsigned long long), st);
   cudaEventRecord(c->tev[0], st);
-  sort_particles(c, x, n, f);
+  sort_particles(c, x, n, f, true, (parts & 1) != 0);
   cudaEventRecord(c->tev[1], st);
   if (parts & 1) {
     cudaEventRecord(c->ev_fork, st);
@@ -482,7 +482,7 @@ p3m_status forces_impl(p3m_ctx* c, const double* x, int64_t n, double* f, double
 
 // out = (dF/dx)^T w
 p3m_status vjp_impl(p3m_ctx* c, const double* x, int64_t n, const double* w, double* out) {
-  sort_particles(c, x, n, out);
+  sort_particles(c, x, n, out, false, false);
   launch_pp_vjp(c, n, w, c->work);  // acc = short-range part
   launch_zero_block(c);
   launch_deposit(c, n);
@@ -696,6 +696,7 @@ p3m_status p3m_create(const p3m_params* params, int64_t n_max, void* stream, p3m
   }
   *c->err_host = 0;
   cudaMemsetAsync(c->err_dev, 0, sizeof(int), c->work);
+  cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * c->nkeys, c->work);
   cudaMemsetAsync(c->qpad, 0, es * c->n_real, c->work);
   cudaMemsetAsync(c->qhat, 0, 2 * es * c->n_cplx, c->work);  // planes z >= n_z stay zero
   if (c->fp32) {
@@ -793,7 +794,7 @@ p3m_status p3m_deposit(p3m_ctx* c, const double* x, int64_t n) {
   p3m_status s = take_deferred(c);
   if (s != P3M_OK) return s;
   if ((s = check_n(c, n)) != P3M_OK) return s;
-  sort_particles(c, x, n, nullptr);
+  sort_particles(c, x, n, nullptr, false, false);
   launch_zero_block(c);
   launch_deposit(c, n);
   c->deposited = true;

@@ -342,8 +342,10 @@ namespace p3m {
 // ---- launch helpers (defined in the .cu files) ----
 // binning and sort (sort.cu)
 void launch_bin(const p3m_ctx* c, const double* x, int64_t n, double* f_zero);
-void launch_scan(const p3m_ctx* c);
-void launch_scatter(const p3m_ctx* c, const double* x, int64_t n);
+// evaluation: also clears the energy and pair accumulators of a force evaluation
+void launch_scan(const p3m_ctx* c, bool evaluation);
+// clear_pp: also clears the FP32 short range's result arrays
+void launch_scatter(const p3m_ctx* c, const double* x, int64_t n, bool clear_pp);
 
 // mesh (pm.cu)
 cudaError_t build_green(p3m_ctx* c);

@@ -50,7 +50,7 @@ struct Acc2 {
 // the sort placed a particle, so no particle within distance 1 is left out.
 template <typename T, typename V>
 __device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restrict__ starts, T px,
-                                         T py, T pz, V&& visit) {
+                                         T py, T pz, int part, int parts, V&& visit) {
   const T slack = static_cast<T>(g.slack);
   const T cwy = static_cast<T>(g.cw[1]), cwz = static_cast<T>(g.cw[2]);
   const T iwx = static_cast<T>(g.inv_cw[0]), iwy = static_cast<T>(g.inv_cw[1]),
@@ -59,10 +59,12 @@ __device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restri
   const int y1 = min(static_cast<int>(floor((py + T(1) + slack) * iwy)), g.nc[1] - 1);
   const int z0 = max(static_cast<int>(floor((pz - T(1) - slack) * iwz)), 0);
   const int z1 = min(static_cast<int>(floor((pz + T(1) + slack) * iwz)), g.nc[2] - 1);
+  int turn = 0;
   for (int rz = z0; rz <= z1; ++rz) {
     const T zl = static_cast<T>(rz) * cwz, zh = zl + cwz;
     const T dz = max((pz < zl ? zl - pz : (pz > zh ? pz - zh : T(0))) - slack, T(0));
     for (int ry = y0; ry <= y1; ++ry) {
+      if ((turn++ & (parts - 1)) != part) continue;
       const T yl = static_cast<T>(ry) * cwy, yh = yl + cwy;
       const T dy = max((py < yl ? yl - py : (py > yh ? py - yh : T(0))) - slack, T(0));
       const T d2 = dy * dy + dz * dz;
@@ -115,6 +117,11 @@ __device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restri
 // ------------------------------------------------------------------------------------------
 constexpr int kPpThreads = 128;     // threads per block of the FP32 short range
 constexpr int kPpBlocksPerSm = 6;    // resident blocks per SM of the short range (80 registers)
+// Lanes that share a pair of particles and split its half-shell rows: 1, doubled (to 16 at most)
+// while the lanes would not fill the resident blocks. Short range with 1, 2, 4, 8, 16 lanes:
+// 5003 particles 308, 183, 126, 89, 73 us; 131,072 (dense) 3.57, 2.70, 1.88, 1.95, 2.00 ms;
+// 261,121 (sphere) 184, 155, 156, 175, 214 us; 2,097,152 748 us (1), 846, 949 (2, 4).
+constexpr int kPpMaxLogParts = 4;
 constexpr int kVjpBlocksPerSm = 10;  // resident blocks per SM of its adjoint (48 registers)
 
 // One 32-byte record (hi and lo float4) in a single 256-bit load through the read-only path.
@@ -269,14 +276,14 @@ __device__ __forceinline__ void pair_poly(const PairPoly& P, float r2, float& fc
 // b's own runs (particle ib in row row_b), for a lane whose two particles sit in different rows
 template <int kRows, typename Emit>
 __device__ __forceinline__ void b_runs(const Geom& g, const uint32_t* __restrict__ starts,
-                                       const float4& pb, const float4& lb, uint32_t ib,
-                                       Emit&& emit) {
+                                       const float4& pb, const float4& lb, uint32_t ib, int part,
+                                       int parts, Emit&& emit) {
   constexpr int kFirst = Rows<kRows>::first, kLast = Rows<kRows>::last;  // half shell
   const uint32_t row_b = __float_as_uint(lb.w) & kRowMask;
   const int cyb = static_cast<int>(row_b % static_cast<uint32_t>(g.nc[1]));
   const int czb = static_cast<int>(row_b / static_cast<uint32_t>(g.nc[1]));
 #pragma unroll 1
-  for (int r = kFirst; r < kLast; ++r) {
+  for (int r = kFirst + part; r < kLast; r += parts) {
     uint32_t j0, j1;
     row_range<kRows>(g, starts, pb.x, pb.y, pb.z, cyb, czb, r, j0, j1);
     j0 = max(j0, ib + 1);
@@ -288,12 +295,13 @@ __device__ __forceinline__ void b_runs(const Geom& g, const uint32_t* __restrict
 // in walk order: emit(j0, j1) for each non-empty run. With a and b in one row (same) each run is
 // the hull of the two particles' runs in one neighbour row and is tested against both;
 // otherwise a's runs come first (split of them) and are tested against a only, then b's
-// (unless kOnlyA: the caller then takes b's runs later, from b_runs).
+// (unless kOnlyA: the caller then takes b's runs later, from b_runs). Of the half shell's rows the
+// lane takes every parts-th from row number part on (lanes that share a pair split its rows).
 template <int kRows, bool kOnlyA = false, typename Emit>
 __device__ __forceinline__ void pair_runs(const Geom& g, const uint32_t* __restrict__ starts,
                                           const float4& pa, const float4& la, const float4& pb,
-                                          const float4& lb, uint32_t ia, bool alive_b, bool& same,
-                                          int& split, Emit&& emit) {
+                                          const float4& lb, uint32_t ia, bool alive_b, int part,
+                                          int parts, bool& same, int& split, Emit&& emit) {
   constexpr int kFirst = Rows<kRows>::first, kLast = Rows<kRows>::last;  // half shell
   const uint32_t ib = ia + 1;
   const uint32_t row_a = __float_as_uint(la.w) & kRowMask;
@@ -303,7 +311,7 @@ __device__ __forceinline__ void pair_runs(const Geom& g, const uint32_t* __restr
   const int cza = static_cast<int>(row_a / static_cast<uint32_t>(g.nc[1]));
   int n = 0;
 #pragma unroll 1
-  for (int r = kFirst; r < kLast; ++r) {
+  for (int r = kFirst + part; r < kLast; r += parts) {
     uint32_t j0, j1;
     row_range<kRows>(g, starts, pa.x, pa.y, pa.z, cya, cza, r, j0, j1);
     j0 = max(j0, ia + 1);  // own row: only the particles after a (a no-op for later rows)
@@ -322,7 +330,7 @@ __device__ __forceinline__ void pair_runs(const Geom& g, const uint32_t* __restr
     }
   }
   split = n;
-  if (!kOnlyA && !same) b_runs<kRows>(g, starts, pb, lb, ib, emit);
+  if (!kOnlyA && !same) b_runs<kRows>(g, starts, pb, lb, ib, part, parts, emit);
 }
 
 // Run slots per lane of k_pp_f32: a's and b's runs, up to twice the half shell when their rows
@@ -355,14 +363,74 @@ __device__ __forceinline__ float4 shfl_f4(float4 v, int src) {
   return v;
 }
 
+// Pairs with images (pp_bc), for the particles less than r_c above the cathode: image pairs act on
+// the particle only. A kernel of its own, since inside k_pp_f32 its registers would spill those of
+// the walk (0 -> 20 bytes; 801 -> 820 us on the 2M sphere). The sort is z-major, so these particles
+// are among the first `near` sorted ones; kImgLanes lanes share one and split the rows around its
+// image point.
+constexpr int kImgLanes = 8;
+
+template <int kDeg>
+__global__ void __launch_bounds__(kThreads)
+    k_pp_images(Geom g, PairPoly P, uint32_t near_cell, const float4* __restrict__ rec,
+                const uint32_t* __restrict__ starts, float4* __restrict__ fpp,
+                float2* __restrict__ flo, float4* __restrict__ fbig, double* __restrict__ energy,
+                unsigned long long* __restrict__ pairs) {
+  const uint32_t near = starts[near_cell];
+  const int part = threadIdx.x & (kImgLanes - 1);
+  const float ch = static_cast<float>(g.img_c);
+  const float cl = static_cast<float>(g.img_c - static_cast<double>(ch));
+  double e_acc = 0.0;
+  unsigned long long ni = 0;
+  for (uint32_t i = (blockIdx.x * kThreads + threadIdx.x) / kImgLanes; i < near;
+       i += gridDim.x * (kThreads / kImgLanes)) {
+    const float4 p = rec[2 * i], l = rec[2 * i + 1];
+    const double zi = static_cast<double>(p.z) + static_cast<double>(l.z);
+    if (zi - 0.5 * g.img_c >= 1.0) continue;
+    const float mz = static_cast<float>(g.img_c - zi);
+    Acc2 sum[3];
+    for (int c = 0; c < 3; ++c) sum[c].hi = sum[c].lo = 0.f;
+    for_rows<float>(g, starts, p.x, p.y, mz, part, kImgLanes, [&](uint32_t ja, uint32_t jb) {
+      float rowv[4] = {0.f, 0.f, 0.f, 0.f};
+      for (uint32_t jj = ja; jj < jb; ++jj) {
+        const float4 hj = rec[2 * jj], lj = rec[2 * jj + 1];
+        const float ax = (p.x - hj.x) + (l.x - lj.x);
+        const float ay = (p.y - hj.y) + (l.y - lj.y);
+        const float s = p.z + hj.z;
+        const float bp = s - p.z;
+        const float e = (p.z - (s - bp)) + (hj.z - bp);
+        const float az = ((s - ch) + e) + ((l.z + lj.z) - cl);
+        const float r2 = ax * ax + ay * ay + az * az;
+        if (r2 < 1.f && r2 > 0.f) {
+          float fco, pot;
+          pair_poly<kDeg>(P, r2, fco, pot);
+          rowv[0] -= fco * ax;
+          rowv[1] -= fco * ay;
+          rowv[2] -= fco * az;
+          rowv[3] -= pot;
+          ++ni;
+        }
+      }
+      for (int c = 0; c < 3; ++c) sum[c].add(rowv[c]);
+      e_acc += static_cast<double>(rowv[3]);
+    });
+    split_add_v4(fpp + i, flo + i, fbig + i, sum[0].hi, sum[1].hi, sum[2].hi, sum[0].lo, sum[1].lo,
+                 sum[2].lo);
+  }
+  block_reduce_add<kThreads>(e_acc, energy);
+  warp_add_u64(ni, pairs + 1);
+}
+
 template <int kDeg, int kRows>
 __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
     k_pp_f32(Geom g, PairPoly P, const uint32_t* __restrict__ total,
              const float4* __restrict__ rec, const uint32_t* __restrict__ starts,
              float4* __restrict__ fpp, float2* __restrict__ flo, float4* __restrict__ fbig,
-             uint32_t* __restrict__ next_tile,
+             uint32_t* __restrict__ next_tile, int log_parts,
              double* __restrict__ energy, unsigned long long* __restrict__ pairs) {
-  constexpr uint32_t kTile = 2 * kPpThreads;  // particles per tile
+  // particles per tile: two a lane, or two for the 2^log_parts lanes that share a pair's rows
+  const uint32_t kTile = (2 * kPpThreads) >> log_parts;
+  const int parts = 1 << log_parts, part = threadIdx.x & (parts - 1);
   constexpr bool kPhased = kRows >= 3;
   constexpr int kPairRuns = pp_pair_runs(kRows);
   static_assert(kPairRuns == (kPhased ? 1 : 2) * Rows<kRows>::half, "run slots");
@@ -376,7 +444,7 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
   const int lane = tid & 31;
   const uint32_t N = *total;
   double e_acc = 0.0;
-  unsigned long long np = 0, ni = 0;
+  unsigned long long np = 0;
   // persistent blocks: each takes the next tile of kTile sorted particles until none is left
   // (the block's four warps work on adjacent particles, which share most of their neighbours
   // in L1)
@@ -387,7 +455,7 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
     __syncthreads();
     if (static_cast<uint64_t>(tile) * kTile >= N) break;
     // the pair the lane holds: a = ia, b = ia + 1 (a thief adopts another lane's pair)
-    uint32_t ia = tile * kTile + 2 * tid;
+    uint32_t ia = tile * kTile + 2 * (tid >> log_parts);
     bool alive_a = ia < N, alive_b = ia + 1 < N;
     // lanes past the last particle read record 0 (in bounds) and take part in the lockstep
     // loop with every result masked out
@@ -405,7 +473,8 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
       ++cnt;
     };
     if (alive_a)
-      pair_runs<kRows, kPhased>(g, starts, pa, la, pb, lb, ia, alive_b, same, split, emit);
+      pair_runs<kRows, kPhased>(g, starts, pa, la, pb, lb, ia, alive_b, part, parts, same, split,
+                                emit);
     bool pending_b = kPhased && alive_a && !same;
     uint32_t ptr = 0, end = 0;
     int k = 0;
@@ -419,44 +488,6 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
     for (int c = 0; c < 4; ++c) sa[c].hi = sa[c].lo = sb[c].hi = sb[c].lo = 0.f;
     float qa[4] = {0.f, 0.f, 0.f, 0.f}, qb[4] = {0.f, 0.f, 0.f, 0.f};
     uint32_t np_part = 0;
-    // images within r_c of particles less than r_c above the cathode (rare): plain loop over
-    // all rows around the image point; image pairs act on the particle only. Taken before the
-    // walk, for the lane's own pair; their potential goes straight to the energy (once)
-    auto images = [&](const float4 pi, const float4 li, Acc2* sum) {
-      const double zi = static_cast<double>(pi.z) + static_cast<double>(li.z);
-      if (zi - 0.5 * g.img_c >= 1.0) return;
-      const float mz = static_cast<float>(g.img_c - zi);
-      const float ch = static_cast<float>(g.img_c);
-      const float cl = static_cast<float>(g.img_c - static_cast<double>(ch));
-      for_rows<float>(g, starts, pi.x, pi.y, mz, [&](uint32_t ja, uint32_t jb) {
-        float rowv[4] = {0.f, 0.f, 0.f, 0.f};
-        for (uint32_t jj = ja; jj < jb; ++jj) {
-          const float4 hj = rec[2 * jj], lj = rec[2 * jj + 1];
-          const float ax = (pi.x - hj.x) + (li.x - lj.x);
-          const float ay = (pi.y - hj.y) + (li.y - lj.y);
-          const float s = pi.z + hj.z;
-          const float bp = s - pi.z;
-          const float e = (pi.z - (s - bp)) + (hj.z - bp);
-          const float az = ((s - ch) + e) + ((li.z + lj.z) - cl);
-          const float r2 = ax * ax + ay * ay + az * az;
-          if (r2 < 1.f && r2 > 0.f) {
-            float fco, pot;
-            pair_poly<kDeg>(P, r2, fco, pot);
-            rowv[0] -= fco * ax;
-            rowv[1] -= fco * ay;
-            rowv[2] -= fco * az;
-            rowv[3] -= pot;
-            ++ni;
-          }
-        }
-        for (int c = 0; c < 3; ++c) sum[c].add(rowv[c]);
-        e_acc += static_cast<double>(rowv[3]);
-      });
-    };
-    if (g.pp_bc) {
-      if (alive_a) images(pa, la, sa);
-      if (alive_b) images(pb, lb, sb);
-    }
     // the held pair's sums (hi + lo of the compensated accumulators) to its force arrays, split
     // like the reactions, and zeroed; sum_i phi_i over ordered pairs takes each unordered
     // pair's potential twice
@@ -544,7 +575,7 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
         if (__any_sync(0xffffffffu, go)) {
           if (go) {
             cnt = 0;
-            b_runs<kRows>(g, starts, pb, lb, ia + 1, emit);
+            b_runs<kRows>(g, starts, pb, lb, ia + 1, part, parts, emit);
             k = 0;
             pending_b = false;
             ta = false;
@@ -641,7 +672,6 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
   }
   if (energy) block_reduce_add<kPpThreads>(e_acc, energy);
   warp_add_u64(2ull * np, pairs);
-  warp_add_u64(ni, pairs + 1);
 }
 
 // (particle, record) distance tests k_pp_f32 makes on the current sorted records: the same
@@ -663,7 +693,7 @@ __global__ void k_pp_count_f32(Geom g, const uint32_t* __restrict__ total,
     const float4 pb = rec[2 * eb], lb = rec[2 * eb + 1];
     bool same = true;
     int split = 0;
-    pair_runs<kRows>(g, starts, pa, la, pb, lb, ia, alive_b, same, split,
+    pair_runs<kRows>(g, starts, pa, la, pb, lb, ia, alive_b, 0, 1, same, split,
                      [&](uint32_t j0, uint32_t j1) { n += j1 - j0; });
     if (same && alive_b) n *= 2;
   }
@@ -796,7 +826,7 @@ __global__ void __launch_bounds__(kThreads, kVjpBlocksPerSm)
         const float mz = static_cast<float>(g.img_c - zi);
         const float ch = static_cast<float>(g.img_c);
         const float cl = static_cast<float>(g.img_c - static_cast<double>(ch));
-        for_rows<float>(g, starts, pi.x, pi.y, mz, [&](uint32_t ja, uint32_t jb) {
+        for_rows<float>(g, starts, pi.x, pi.y, mz, 0, 1, [&](uint32_t ja, uint32_t jb) {
           float rowv[3] = {0.f, 0.f, 0.f};
           for (uint32_t jj = ja; jj < jb; ++jj) {
             const float4 hj = rec[2 * jj], lj = rec[2 * jj + 1];
@@ -846,16 +876,17 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
   }
   const uint32_t* total = c->starts + c->nkeys;
   {
-    // the kernel adds each pair's force to both particles: the result (coarse, fine and big
-    // parts) starts at zero
+    // the kernel adds each pair's force to both particles; the result (coarse, fine and big parts)
+    // and the tile counter were cleared by the sort
     float4* fbig = c->fplo + c->n_max;
-    cudaMemsetAsync(c->fpp, 0, sizeof(float4) * static_cast<size_t>(n), s);
-    cudaMemsetAsync(c->fplo, 0, sizeof(float2) * static_cast<size_t>(n), s);
-    cudaMemsetAsync(fbig, 0, sizeof(float4) * static_cast<size_t>(n), s);
-    cudaMemsetAsync(c->pp_tile, 0, sizeof(uint32_t), s);
     // persistent grid of a few blocks per SM: the SM resources it leaves free let the mesh
     // chain, on the other stream, run at the same time
-    const int64_t tiles = (n + 2 * kPpThreads - 1) / (2 * kPpThreads);  // two particles a thread
+    // lanes per pair of particles (kPpMaxLogParts)
+    const int64_t full = static_cast<int64_t>(kPpBlocksPerSm) * c->num_sms * kPpThreads;
+    int log_parts = 0;
+    while (log_parts < kPpMaxLogParts && (((n + 1) / 2) << log_parts) < full) ++log_parts;
+    const int64_t per_tile = (2 * kPpThreads) >> log_parts;
+    const int64_t tiles = (n + per_tile - 1) / per_tile;
     const unsigned wblocks = static_cast<unsigned>(
         std::min<int64_t>(tiles, static_cast<int64_t>(kPpBlocksPerSm) * c->num_sms));
     // the kernel for the context's row geometry (Geom::rows cell rows per cutoff)
@@ -868,8 +899,37 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
       kern<<<wblocks, kPpThreads, smem, s>>>(
           c->g, c->poly, total, static_cast<const float4*>(c->recp), c->starts,
           static_cast<float4*>(c->fpp), reinterpret_cast<float2*>(c->fplo), fbig, c->pp_tile,
-          c->energy_acc, c->pair_acc);
+          log_parts, c->energy_acc, c->pair_acc);
     };
+    if (c->g.pp_bc) {
+      // every particle less than r_c above the cathode lies in a z row below this cell
+      const double top = (0.5 * c->g.img_c + 1.0 + c->g.slack) * c->g.inv_cw[2];
+      const int rows = std::max(0, std::min(c->g.nc[2], static_cast<int>(std::floor(top)) + 1));
+      const uint32_t near_cell = static_cast<uint32_t>(rows) * c->g.nc[1] * c->g.nc[0];
+      const unsigned iblocks = static_cast<unsigned>(std::min<int64_t>(
+          (n * kImgLanes + kThreads - 1) / kThreads, static_cast<int64_t>(c->num_sms) * 8));
+      auto images = [&](auto kern) {
+        kern<<<iblocks, kThreads, 0, s>>>(c->g, c->poly, near_cell,
+                                          static_cast<const float4*>(c->recp), c->starts,
+                                          static_cast<float4*>(c->fpp),
+                                          reinterpret_cast<float2*>(c->fplo), fbig,
+                                          c->energy_acc, c->pair_acc);
+      };
+      switch (c->poly.deg) {
+        case 4: images(k_pp_images<4>); break;
+        case 5: images(k_pp_images<5>); break;
+        case 6: images(k_pp_images<6>); break;
+        case 7: images(k_pp_images<7>); break;
+        case 8: images(k_pp_images<8>); break;
+        case 9: images(k_pp_images<9>); break;
+        case 10: images(k_pp_images<10>); break;
+        case 11: images(k_pp_images<11>); break;
+        case 12: images(k_pp_images<12>); break;
+        case 13: images(k_pp_images<13>); break;
+        case 14: images(k_pp_images<14>); break;
+        default: images(k_pp_images<15>); break;
+      }
+    }
     switch (c->poly.deg) {
       case 4: run(k_pp_f32<4, 1>, k_pp_f32<4, 2>, k_pp_f32<4, 3>); break;
       case 5: run(k_pp_f32<5, 1>, k_pp_f32<5, 2>, k_pp_f32<5, 3>); break;

@@ -463,7 +463,6 @@ void run64(const p3m_ctx* c, int64_t n, Args64 a, cudaStream_t s) {
   const int64_t warps = ((n << a.log_s) + 31) / 32;
   const unsigned blocks = static_cast<unsigned>(
       std::min<int64_t>((warps + kWarps64 - 1) / kWarps64, c->num_sms));
-  cudaMemsetAsync(c->pp_tile, 0, sizeof(uint32_t), s);
   kern<<<blocks, kThreads64, smem, s>>>(c->g, a);
 }
 

@@ -12,6 +12,13 @@ namespace p3m {
 namespace {
 
 constexpr int kBinThreads = 256;
+// what the second scan pass clears for the kernels after the sort
+struct SortClear {
+  uint32_t* tile;              // the short range's tile counter
+  double* energy;              // [2]
+  unsigned long long* pairs;   // [3]
+};
+
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;  // per thread
 constexpr int kScanTile = kScanThreads * kScanItems;
@@ -137,9 +144,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t* __r
 // total to out_total.
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* __restrict__ bsum,
                                                             uint64_t nb,
-                                                            uint32_t* __restrict__ out_total) {
+                                                            uint32_t* __restrict__ out_total,
+                                                            SortClear clear) {
   __shared__ uint32_t warp_tot[kScanThreads / 32];
   __shared__ uint32_t carry_s;
+  // the accumulators of the evaluation that follows (null: left alone)
+  if (threadIdx.x == 0) *clear.tile = 0;
+  if (clear.energy && threadIdx.x < 2) clear.energy[threadIdx.x] = 0.0;
+  if (clear.pairs && threadIdx.x < 3) clear.pairs[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) carry_s = 0;
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -174,19 +186,32 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* __restrict
   if (threadIdx.x == 0) *out_total = carry_s;
 }
 
+// Level 3: the tiles' offsets; and the counts back to zero for the next sort.
 __global__ void k_scan_add(uint32_t* __restrict__ out, const uint32_t* __restrict__ bsum,
-                           uint64_t n) {
+                           uint32_t* __restrict__ counts, uint64_t n) {
   const uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
-  if (i < n) out[i] += bsum[i / kScanTile];
+  if (i >= n) return;
+  out[i] += bsum[i / kScanTile];
+  counts[i] = 0u;
 }
 
 template <bool kFP32>
 __global__ void k_scatter(Geom g, const double* __restrict__ x, int64_t n,
                           uint32_t* __restrict__ keys, const uint32_t* __restrict__ ranks,
                           const uint32_t* __restrict__ starts, void* __restrict__ recp,
-                          void* __restrict__ recm, int64_t n_max) {
+                          void* __restrict__ recm, int64_t n_max, float4* __restrict__ fpp,
+                          float4* __restrict__ fplo) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= n) return;
+  if constexpr (kFP32) {
+    // the FP32 short range adds into its result arrays: cleared here (entry i, coalesced) rather
+    // than by three memsets before it
+    if (fpp) {
+      fpp[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      reinterpret_cast<float2*>(fplo)[i] = make_float2(0.f, 0.f);
+      fplo[n_max + i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
   const uint32_t key = keys[i];
   if (key == kInvalidKey) return;
   const uint32_t pos = starts[key] + ranks[i];
@@ -303,30 +328,35 @@ inline unsigned grid_for(int64_t n, int threads) {
 }  // namespace
 
 void launch_bin(const p3m_ctx* c, const double* x, int64_t n, double* f_zero) {
-  cudaMemsetAsync(c->counts, 0, sizeof(uint32_t) * c->nkeys, c->work);
-  if (n == 0) return;
+  if (n == 0) return;  // the counts are zero: cleared at creation and after every scan
   k_bin<<<grid_for(n, kBinThreads), kBinThreads, 0, c->work>>>(c->g, x, n, c->counts, c->keys,
                                                                   c->ranks, c->err_dev, f_zero);
 }
 
-void launch_scan(const p3m_ctx* c) {
+void launch_scan(const p3m_ctx* c, bool evaluation) {
   const uint64_t n = c->nkeys;
   const uint64_t tiles = (n + kScanTile - 1) / kScanTile;
   k_scan_tiles<<<static_cast<unsigned>(tiles), kScanThreads, 0, c->work>>>(c->counts, c->starts,
                                                                              c->bsum, n);
-  k_scan_sums<<<1, kScanThreads, 0, c->work>>>(c->bsum, tiles, c->starts + n);
+  SortClear clear{c->pp_tile, nullptr, nullptr};
+  if (evaluation) {
+    clear.energy = c->energy_acc;
+    clear.pairs = c->pair_acc;
+  }
+  k_scan_sums<<<1, kScanThreads, 0, c->work>>>(c->bsum, tiles, c->starts + n, clear);
   k_scan_add<<<static_cast<unsigned>((n + 255) / 256), 256, 0, c->work>>>(c->starts, c->bsum,
-                                                                            n);
+                                                                            c->counts, n);
 }
 
-void launch_scatter(const p3m_ctx* c, const double* x, int64_t n) {
+void launch_scatter(const p3m_ctx* c, const double* x, int64_t n, bool clear_pp) {
   if (n == 0) return;
   if (c->fp32)
     k_scatter<true><<<grid_for(n, kBinThreads), kBinThreads, 0, c->work>>>(
-        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max);
+        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max,
+        clear_pp ? static_cast<float4*>(c->fpp) : nullptr, c->fplo);
   else {
     k_scatter<false><<<grid_for(n, kBinThreads), kBinThreads, 0, c->work>>>(
-        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max);
+        c->g, x, n, c->keys, c->ranks, c->starts, c->recp, c->recm, c->n_max, nullptr, nullptr);
     if (c->det)
       k_cell_order<<<static_cast<unsigned>((c->nkeys + kBinThreads - 1) / kBinThreads),
                      kBinThreads, 0, c->work>>>(c->nkeys, c->starts, static_cast<float4*>(c->recp),

@@ -804,3 +804,24 @@ def test_fp64_lane_groups(n, rows):
     assert pairs == (ref.pairs, ref.image_pairs)
     assert rel(f, ref.F) <= TOL[0]
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [2, 3, 255, 14591, 14592, 29185, 58367, 116737, 233472])
+def test_fp32_lanes_sharing_a_pair(n):
+    # FP32 short range: from one lane per pair of particles (233,472 particles and more fill the
+    # resident blocks) to 16 lanes that split the pair's rows, on both sides of every change: the
+    # same pairs, images and forces. The cutoff shrinks with the count, so that the oracle's sum
+    # stays small.
+    x = np.random.default_rng(n).uniform(-1e-3, 1e-3, size=(n, 3))
+    x[:, 2] += 1.02e-3
+    box = np.array([[-1e-3, -1e-3, 0.0], [1e-3, 1e-3, 2.04e-3]])
+    P = O.auto_mesh(box, 32, rc_over_h=1.0 if n > 20000 else 2.0, pm_bc=1, pp_bc=1, z_cathode=0.0)
+    ref = O.forces(x, P)
+    ctx = p3m().Context(gpu_params(P, 1), n)
+    f = ctx.forces(cuda(x))
+    pairs = ctx.pair_count()
+    ctx.sync()
+    assert abs(pairs[0] - ref.pairs) <= 2 + 2e-7 * ref.pairs
+    assert abs(pairs[1] - ref.image_pairs) <= 2
+    assert rel(f, ref.F) <= TOL[1]
+    ctx.close()
