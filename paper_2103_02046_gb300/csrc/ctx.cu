@@ -287,7 +287,7 @@ void free_all(p3m_ctx* c) {
                   c->acc, c->qpad, c->qhat, c->qhat2, c->khat_f, c->khat_i, c->fhat, c->freal,
                   c->phihat, c->phireal, c->dfac, c->ztw, c->box_real, c->box_spec, c->box_mult,
                   c->energy_acc, c->pair_acc,
-                  c->pp_tile, c->err_dev, c->ckpt, c->seg, c->lam_x, c->lam_p, c->xw, c->pw,
+                  c->pp_tile, c->dense_flags, c->dense_tiles, c->err_dev, c->ckpt, c->seg, c->lam_x, c->lam_p, c->xw, c->pw,
                   c->tmp3, c->tmp3b, c->f_work, c->red, c->ered, c->q128, c->dbound, c->dred};
   for (void* b : bufs) cudaFree(b);
   if (c->err_host) cudaFreeHost(c->err_host);
@@ -453,6 +453,7 @@ p3m_status forces_impl(p3m_ctx* c, const double* x, int64_t n, double* f, double
   sort_particles(c, x, n, f, true, (parts & 1) != 0);
   cudaEventRecord(c->tev[1], st);
   if (parts & 1) {
+    if (c->fp32) launch_dense_tiles(c, n, st);
     cudaEventRecord(c->ev_fork, st);
     cudaStreamWaitEvent(c->s_pp, c->ev_fork, 0);
     cudaEventRecord(c->tev[6], c->s_pp);
@@ -642,7 +643,11 @@ p3m_status p3m_create(const p3m_params* params, int64_t n_max, void* stream, p3m
   }
   A(alloc(&c->energy_acc, 2));
   A(alloc(&c->pair_acc, 3));
-  A(alloc(&c->pp_tile, 1));
+  A(alloc(&c->pp_tile, 3));
+  if (c->fp32) {
+    A(alloc(&c->dense_flags, n_max / 64 + 1));
+    A(alloc(&c->dense_tiles, 2 * (n_max / 64 + 1)));
+  }
   A(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
   A(alloc(&c->err_dev, 1));
   A(alloc(&c->red, 32));

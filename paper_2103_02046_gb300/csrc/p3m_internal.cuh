@@ -306,7 +306,11 @@ struct p3m_ctx {
   // diagnostics
   double* energy_acc = nullptr;              // device [2]
   unsigned long long* pair_acc = nullptr;    // device [3]: pairs, image pairs, candidates
-  uint32_t* pp_tile = nullptr;               // device [1]: next tile of the persistent short range
+  // device [3], zeroed by every sort: next tile of the persistent short range; number of dense
+  // tiles; next item of the dense tiles
+  uint32_t* pp_tile = nullptr;
+  uint32_t* dense_flags = nullptr;           // FP32: [n_max / 64 + 1] which particles the tiles hold
+  uint2* dense_tiles = nullptr;              // FP32: [2 (n_max / 64 + 1)] first particle, count
   int num_sms = 0;
   int* err_dev = nullptr;                    // device error bits
   int* err_host = nullptr;                   // pinned mirror of err_dev
@@ -377,6 +381,13 @@ void launch_get_mesh(const p3m_ctx* c, int which, double* out);
 // want_energy: the short-range energy is asked for (the FP64 path skips the pair potentials
 // otherwise)
 void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy);
+// dense regions (pp_dense.cu): the list of tiles and the flags of the particles they hold, after
+// the sort; the tiles' short range (the walk leaves those particles out); the flags, or nullptr if
+// a bunch of n particles has no tiles
+void launch_dense_tiles(const p3m_ctx* c, int64_t n, cudaStream_t s);
+void launch_pp_dense(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy);
+const uint32_t* dense_flags(const p3m_ctx* c, int64_t n);
+void launch_pp_dense_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaStream_t s);
 // (particle, record) distance tests of the FP32 short range on the current sorted records,
 // into *out (FP64 contexts: nothing; their short range counts as it runs)
 void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaStream_t s);

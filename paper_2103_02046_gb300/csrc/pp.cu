@@ -23,25 +23,12 @@
 #include <cmath>
 #include <type_traits>
 
-#include "pp_common.cuh"
+#include "pp_f32.cuh"
 
 namespace p3m {
 namespace {
 
 constexpr int kThreads = 128;
-
-// two-float accumulator (hi + lo) with Knuth's TwoSum
-struct Acc2 {
-  float hi, lo;
-  __device__ __forceinline__ void add(float v) {
-    const float s = hi + v;
-    const float bp = s - hi;
-    const float err = (hi - (s - bp)) + (v - bp);
-    hi = s;
-    lo += err;
-  }
-  __device__ __forceinline__ float value() const { return hi + lo; }
-};
 
 // Calls visit(j0, j1) for every neighbour row of the query point (px, py, pz) (cutoff units)
 // that can hold particles within distance 1, with [j0, j1) the sorted range of its cells whose
@@ -123,133 +110,6 @@ constexpr int kPpBlocksPerSm = 6;    // resident blocks per SM of the short rang
 // 261,121 (sphere) 184, 155, 156, 175, 214 us; 2,097,152 748 us (1), 846, 949 (2, 4).
 constexpr int kPpMaxLogParts = 4;
 constexpr int kVjpBlocksPerSm = 10;  // resident blocks per SM of its adjoint (48 registers)
-
-// One 32-byte record (hi and lo float4) in a single 256-bit load through the read-only path.
-// The records array is 32-byte aligned and not written while the short range runs.
-__device__ __forceinline__ void load_rec32(const float4* p, float4& h, float4& l) {
-  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=f"(h.x), "=f"(h.y), "=f"(h.z), "=f"(h.w), "=f"(l.x), "=f"(l.y), "=f"(l.z), "=f"(l.w)
-      : "l"(p));
-}
-
-__device__ __forceinline__ void red_add_v4(float4* dst, float a, float b, float c, float d) {
-  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(a), "f"(b),
-               "f"(c), "f"(d)
-               : "memory");
-}
-
-// predicated form: the reduction happens only where p holds (no branch around it)
-__device__ __forceinline__ void red_add_v4_if(bool p, float4* dst, float a, float b, float c,
-                                              float d) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
-      "@q red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n\t}" ::"l"(dst),
-      "f"(a), "f"(b), "f"(c), "f"(d), "r"(static_cast<int>(p))
-      : "memory");
-}
-
-// Error-free split of a short-range force component about the grid of multiples of
-// kSplitQ = 2^-6 (the kernel's force unit is the pair force at a cutoff length's scale, so the
-// terms are O(1) and a particle's sums stay far below 2^24 kSplitQ even with tens of thousands
-// of neighbours): v = c + f exactly, with c a multiple of kSplitQ and |f| <= kSplitQ / 2.
-// Adding kSplitC = 1.5 * 2^23 * kSplitQ rounds v to that grid (the sum's last mantissa bit is
-// worth kSplitQ); subtracting it again is exact (Sterbenz), and so is v - c. The coarse parts c
-// of one particle's terms are multiples of kSplitQ, so their FP32 atomic sum is exact, and
-// independent of the order, while it stays below 2^24 kSplitQ in magnitude; only the small
-// parts f are rounded when summed.
-constexpr float kSplitQ = 0.015625f;
-constexpr float kSplitC = 1.5f * 8388608.f * kSplitQ;
-// A term of magnitude 2^21 kSplitQ or more (a pair closer than about 0.006 cutoff lengths)
-// would take the coarse sum out of its exact range: it goes whole to a third array (big), where
-// a particle rarely has more than one term.
-constexpr float kBigTerm = 2097152.f * kSplitQ;
-// (in PTX, so that no compiler pass folds (v + C) - C into v)
-__device__ __forceinline__ void split_q(float v, float& c, float& f) {
-  float t;
-  asm("add.rn.f32 %0, %1, %2;" : "=f"(t) : "f"(v), "f"(kSplitC));
-  asm("sub.rn.f32 %0, %1, %2;" : "=f"(c) : "f"(t), "f"(kSplitC));
-  asm("sub.rn.f32 %0, %1, %2;" : "=f"(f) : "f"(v), "f"(c));
-}
-
-__device__ __forceinline__ bool big_term(float a, float b, float c) {
-  return fmaf(a, a, fmaf(b, b, c * c)) >= kBigTerm * kBigTerm;
-}
-
-// 2-wide reduction (the fine x and y parts)
-__device__ __forceinline__ void red_add_v2_if(bool p, float2* dst, float a, float b) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t"
-      "@q red.global.add.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(dst),
-      "f"(a), "f"(b), "r"(static_cast<int>(p))
-      : "memory");
-}
-
-// One particle's short-range force held in three arrays: co (float4: the coarse x, y, z parts and
-// the fine z part), fi (float2: the fine x and y parts) and bg (float4: big terms). Each added
-// term is split; the coarse parts and the fine z part go out in one 4-wide reduction into co, the
-// fine x and y parts in one 2-wide reduction into fi (24 bytes a term; the fourth coarse slot
-// would otherwise carry a zero), or, if the term is big, it is reduced whole into bg. The result
-// is the exact sum up to the rounding of the fine sums, whose terms are at most kSplitQ / 2, and
-// of the (rare) big terms. `big` may be set for terms below kBigTerm too (a cheaper test that
-// never misses a big term).
-__device__ __forceinline__ void split_add_v4_if(bool p, bool big, float4* co, float2* fi,
-                                                float4* bg, float a, float b, float c) {
-  // x and y split on the two-wide FP32 instructions, z on the scalar ones (the same steps)
-  const float2 ab = make_float2(a, b);
-  const float2 abc = __fadd2_rn(__fadd2_rn(ab, make_float2(kSplitC, kSplitC)),
-                                make_float2(-kSplitC, -kSplitC));
-  const float2 abf = __fadd2_rn(ab, make_float2(-abc.x, -abc.y));
-  float cc, cf;
-  split_q(c, cc, cf);
-  red_add_v4_if(p && !big, co, abc.x, abc.y, cc, cf);
-  red_add_v2_if(p && !big, fi, abf.x, abf.y);
-  if (p && big) red_add_v4(bg, abc.x + abf.x, abc.y + abf.y, cc + cf, 0.f);  // (a, b, c); rare
-}
-// the same for a compensated sum hi + lo (lo far below hi): hi is split, lo joins the fine part
-__device__ __forceinline__ void split_add_v4(float4* co, float2* fi, float4* bg, float a, float b,
-                                             float c, float la, float lb, float lc) {
-  if (big_term(a, b, c)) {
-    red_add_v4(bg, a, b, c, 0.f);
-    red_add_v4(co, 0.f, 0.f, 0.f, lc);
-    red_add_v2_if(true, fi, la, lb);
-    return;
-  }
-  float ac, af, bc, bf, cc, cf;
-  split_q(a, ac, af);
-  split_q(b, bc, bf);
-  split_q(c, cc, cf);
-  red_add_v4(co, ac, bc, cc, __fadd_rn(cf, lc));
-  red_add_v2_if(true, fi, __fadd_rn(af, la), __fadd_rn(bf, lb));
-}
-
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float ex2_ftz(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-__device__ __forceinline__ float rcp_ftz(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// R(x) = erfc(x) e^{x^2}, x = kappa rho, as t P(u): t = 1 / (1 + p kappa rho), u = t - t_c
-template <int kDeg, bool kHw>
-__device__ __forceinline__ float erfcx_poly(const PairPoly& P, float rho) {
-  const float t = kHw ? rcp_ftz(fmaf(P.pk, rho, 1.f)) : 1.f / fmaf(P.pk, rho, 1.f);
-  const float u = t - P.tc;
-  float R = P.c[kDeg];
-#pragma unroll
-  for (int m = kDeg - 1; m >= 0; --m) R = fmaf(R, u, P.c[m]);
-  return R * t;
-}
 
 // pair_poly on the hardware approximations; r2 in (0, 1]
 template <int kDeg>
@@ -427,6 +287,7 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
              const float4* __restrict__ rec, const uint32_t* __restrict__ starts,
              float4* __restrict__ fpp, float2* __restrict__ flo, float4* __restrict__ fbig,
              uint32_t* __restrict__ next_tile, int log_parts,
+             const uint32_t* __restrict__ dense,
              double* __restrict__ energy, unsigned long long* __restrict__ pairs) {
   // particles per tile: two a lane, or two for the 2^log_parts lanes that share a pair's rows
   const uint32_t kTile = (2 * kPpThreads) >> log_parts;
@@ -457,6 +318,7 @@ __global__ void __launch_bounds__(kPpThreads, kPpBlocksPerSm)
     // the pair the lane holds: a = ia, b = ia + 1 (a thief adopts another lane's pair)
     uint32_t ia = tile * kTile + 2 * (tid >> log_parts);
     bool alive_a = ia < N, alive_b = ia + 1 < N;
+    if (dense && alive_a && in_dense_tile(dense, ia)) alive_a = alive_b = false;
     // lanes past the last particle read record 0 (in bounds) and take part in the lockstep
     // loop with every result masked out
     const uint32_t ea = alive_a ? ia : 0u, eb = alive_b ? ia + 1 : ea;
@@ -681,12 +543,13 @@ template <int kRows>
 __global__ void k_pp_count_f32(Geom g, const uint32_t* __restrict__ total,
                                const float4* __restrict__ rec,
                                const uint32_t* __restrict__ starts,
+                               const uint32_t* __restrict__ dense,
                                unsigned long long* __restrict__ out) {
   const uint32_t N = *total;
   const uint32_t lane_pair = blockIdx.x * static_cast<uint32_t>(blockDim.x) + threadIdx.x;
   const uint32_t ia = 2 * lane_pair, ib = ia + 1;
   unsigned long long n = 0;
-  if (ia < N) {
+  if (ia < N && !(dense && in_dense_tile(dense, ia))) {
     const bool alive_b = ib < N;
     const uint32_t eb = alive_b ? ib : ia;
     const float4 pa = rec[2 * ia], la = rec[2 * ia + 1];
@@ -879,6 +742,8 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
     // the kernel adds each pair's force to both particles; the result (coarse, fine and big parts)
     // and the tile counter were cleared by the sort
     float4* fbig = c->fplo + c->n_max;
+    // particles with many neighbours go to the tile kernel, the others to the walk
+    const uint32_t* dense = dense_flags(c, n);
     // persistent grid of a few blocks per SM: the SM resources it leaves free let the mesh
     // chain, on the other stream, run at the same time
     // lanes per pair of particles (kPpMaxLogParts)
@@ -899,7 +764,7 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
       kern<<<wblocks, kPpThreads, smem, s>>>(
           c->g, c->poly, total, static_cast<const float4*>(c->recp), c->starts,
           static_cast<float4*>(c->fpp), reinterpret_cast<float2*>(c->fplo), fbig, c->pp_tile,
-          log_parts, c->energy_acc, c->pair_acc);
+          log_parts, dense, c->energy_acc, c->pair_acc);
     };
     if (c->g.pp_bc) {
       // every particle less than r_c above the cathode lies in a z row below this cell
@@ -944,6 +809,8 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
       case 14: run(k_pp_f32<14, 1>, k_pp_f32<14, 2>, k_pp_f32<14, 3>); break;
       default: run(k_pp_f32<15, 1>, k_pp_f32<15, 2>, k_pp_f32<15, 3>); break;
     }
+    // (after the walk: in a sparse bunch the walk is what takes time, and it then starts at once)
+    launch_pp_dense(c, n, s, want_energy);
   }
 }
 
@@ -956,7 +823,9 @@ void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaS
               : c->g.rows == 2 ? k_pp_count_f32<2>
                                : k_pp_count_f32<3>;
   kern<<<static_cast<unsigned>((lane_pairs + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      c->g, c->starts + c->nkeys, static_cast<const float4*>(c->recp), c->starts, out);
+      c->g, c->starts + c->nkeys, static_cast<const float4*>(c->recp), c->starts,
+      dense_flags(c, n), out);
+  launch_pp_dense_count(c, n, out, s);
 }
 
 void launch_pp_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s) {

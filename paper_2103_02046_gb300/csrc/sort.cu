@@ -14,7 +14,7 @@ namespace {
 constexpr int kBinThreads = 256;
 // what the second scan pass clears for the kernels after the sort
 struct SortClear {
-  uint32_t* tile;              // the short range's tile counter
+  uint32_t* tile;              // [3] the short range's counters
   double* energy;              // [2]
   unsigned long long* pairs;   // [3]
 };
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* __restrict
   __shared__ uint32_t warp_tot[kScanThreads / 32];
   __shared__ uint32_t carry_s;
   // the accumulators of the evaluation that follows (null: left alone)
-  if (threadIdx.x == 0) *clear.tile = 0;
+  if (threadIdx.x < 3) clear.tile[threadIdx.x] = 0;
   if (clear.energy && threadIdx.x < 2) clear.energy[threadIdx.x] = 0.0;
   if (clear.pairs && threadIdx.x < 3) clear.pairs[threadIdx.x] = 0ull;
   if (threadIdx.x == 0) carry_s = 0;

@@ -825,3 +825,42 @@ def test_fp32_lanes_sharing_a_pair(n):
     assert abs(pairs[1] - ref.image_pairs) <= 2
     assert rel(f, ref.F) <= TOL[1]
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [32767, 32768, 33001])
+@pytest.mark.parametrize("rows", [1, 2, 3])
+def test_fp32_dense_tiles(n, rows):
+    # FP32 short range with dense and sparse regions in one bunch, on both sides of the count from
+    # which tiles are used: 80% of the particles in a core a cutoff length wide (tiles of 64,
+    # several to a cell row, pieces at row ends), a coincident and two close pairs among them, the
+    # rest spread out (the walk): forces, energy, pair counts with images
+    r = np.random.default_rng(100 * n + rows)
+    k = (4 * n) // 5
+    x = np.concatenate([r.normal(scale=[1.5e-4, 1.3e-4, 1.8e-4], size=(k, 3)),
+                        r.uniform(-1e-3, 1e-3, size=(n - k, 3))])
+    x[1] = x[0]
+    x[3] = x[2] + 1e-6
+    x[5] = x[4] + [4e-7, 0.0, 0.0]
+    x = x[r.permutation(n)]
+    x[:, 2] += 1.02e-3
+    P = O.auto_mesh(np.array([[-1e-3, -1e-3, 0.0], [1e-3, 1e-3, 2.04e-3]]), 32, rc_over_h=2.0,
+                    pm_bc=1, pp_bc=1, z_cathode=0.0)
+    ref = O.forces(x, P)
+    assert ref.pairs > 1000 * n  # a mean of 1000 neighbours and more
+    ctx = p3m().Context(gpu_params(P, 1, search_rows=rows, search_xcells=8), n)
+    f, e = ctx.forces(cuda(x), energy=True)
+    pairs = ctx.pair_count()
+    ncand = ctx.candidate_count()
+    ctx.sync()
+    # pairs whose FP32 r^2 rounds across the cutoff: r^2 carries a few 2^-24, so a shell of that
+    # relative thickness, 1.5 * 4 * 2^-24 of the pairs within
+    assert abs(pairs[0] - ref.pairs) <= 4 + 4e-7 * ref.pairs
+    assert abs(pairs[1] - ref.image_pairs) <= 2
+    assert ref.pairs // 2 <= ncand
+    assert rel(f, ref.F) <= TOL[1]
+    eg = e.cpu().numpy()
+    assert abs(eg[0] - ref.U_pp) <= 1e-5 * abs(ref.U_pp)
+    # without the energy the potentials are left out of the tiles: the same forces
+    assert rel(ctx.forces(cuda(x)), ref.F) <= TOL[1]
+    ctx.sync()
+    ctx.close()
