@@ -218,16 +218,40 @@ __device__ __forceinline__ long long orig_index(const Rec64* recm, uint32_t i) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Charge assignment with a shared-memory tile: a block takes kDepPerBlock consecutive sorted
-// particles (one stretch of an x-row of cells, so their supports overlap heavily), sums their
-// weights into a tile of the mesh covering the block's bounding box, then adds the non-zero tile
-// entries to the mesh with one global atomic each. Blocks whose box does not fit the tile fall
-// back to global atomics per weight.
+// Charge assignment with a shared-memory tile: a block takes consecutive sorted particles (one
+// stretch of an x-row of cells, so their supports overlap heavily), sums their weights into a tile
+// of the mesh covering the block's bounding box, then adds the non-zero tile entries to the mesh
+// with one global atomic each. Blocks whose box does not fit the tile fall back to global atomics
+// per weight.
+//
+// The tile holds fixed-point numbers, because integer shared-memory atomics are native while
+// floating-point ones are compare-and-swap loops: FP32 charges in one 32-bit word, the others in
+// two (FP32 dipoles) or three (FP64) words of 21 bits each, added word by word without carries. At
+// most 1024 particles add to a node, so a word's sum stays below 2^32 (and the signed leading word
+// of a dipole within 2^31). The sums inside a tile are exact and independent of the order.
+//
+// A block holds 256 threads: four particles each from kDepManyParticles on, one each from
+// kDepLanesBelow on; below that eight lanes share a particle (its 9 rows of nodes), so that a few
+// thousand particles still fill the SMs. Deposit stage, four particles a thread / one / shared:
+// 4096 FP64 46 / 21 / 13 us, 5003 FP32 17 / 13 / 11, 261,121 FP32 28 / 22 / 56, 2,097,152 FP32
+// 71 / 99 / 364, FP64 523 / 610 / 1661 (with FP64 compare-and-swap in the tile: 4096 156, 2M 624 us).
+// The FP64 tile is bound by the FP64 unit: weights, 27 products and 27 conversions a particle.
 // ---------------------------------------------------------------------------------------------
 constexpr int kDepThreads = 256;
 constexpr int kDepItems = 4;
-constexpr int kDepPerBlock = kDepThreads * kDepItems;
-constexpr int kTileBytes = 32768;
+constexpr int kShareLanes = 8;
+constexpr int64_t kDepManyParticles = 600000, kDepLanesBelow = 150000;
+
+// words per tile node
+template <typename T, bool kDipole>
+__host__ __device__ constexpr int dep_words() {
+  return sizeof(T) == 8 ? 3 : (kDipole ? 2 : 1);
+}
+// nodes of the tile
+template <typename T>
+__host__ __device__ constexpr int dep_tile() {
+  return sizeof(T) == 8 ? 4096 : 8192;
+}
 
 // The charged block n^3 of the doubled mesh to zero (grid: x-y plane by z plane). As one kernel: a
 // pitched 3D memset of the same block takes 200 us and more, whatever the mesh (measured: the
@@ -240,38 +264,34 @@ __global__ void k_zero_block(Geom g, T* __restrict__ q) {
   q[real_index(g, x, y, blockIdx.y)] = T(0);
 }
 
-template <typename T, bool kDipole>
+template <typename T, bool kDipole, bool kShare>
 __global__ void __launch_bounds__(kDepThreads)
     k_deposit_tiled(Geom g, const uint32_t* __restrict__ total,
                     const typename RecT<T>::type* __restrict__ recm,
                     const typename RecT<T>::type* __restrict__ recp,
-                    const double* __restrict__ w, T* __restrict__ qpad) {
-  // FP32 charge deposit: the tile accumulates in unsigned 32-bit fixed point, because integer
-  // shared-memory atomics are native while float ones are compare-and-swap loops. A tile node
-  // receives at most one weight from each of the block's 1024 particles: at most 27/64 with TSC
-  // (2^23 per unit of weight keeps the sum below 1024 * 27/64 * 2^23 < 2^32) and at most 1 with
-  // CIC (2^21 per unit: below 2^31). Sums inside a tile are then exact and independent of the
-  // order of the particles.
-  constexpr bool kFixed = (sizeof(T) == 4) && !kDipole;
-  using Slot = typename std::conditional<kFixed, unsigned int, T>::type;
-  constexpr int kTile = kTileBytes / sizeof(Slot);
-  __shared__ Slot tile[kTile];
+                    const double* __restrict__ w, T* __restrict__ qpad, int items) {
+  constexpr int kWords = dep_words<T, kDipole>(), kDepTile = dep_tile<T>();
+  constexpr int kMaxExp = sizeof(T) == 8 ? 900 : 80;
+  extern __shared__ uint32_t tile[];  // [kWords][kDepTile], leading word first
   __shared__ int bmin[3], bmax[3];
+  __shared__ unsigned long long wmax;  // kDipole: bits of the largest sum_d |w_d| / h_d
   const uint32_t N = *total;
-  const uint32_t b0 = blockIdx.x * kDepPerBlock;
+  constexpr uint32_t stride = kDepThreads / (kShare ? kShareLanes : 1);  // particles per item
+  const uint32_t b0 = blockIdx.x * (stride * items);
   if (b0 >= N) return;
+  const uint32_t first = b0 + (kShare ? threadIdx.x / kShareLanes : threadIdx.x);
+  const int part = threadIdx.x % kShareLanes;  // kShare: the lane's turn among a particle's
   const int S = g.order == 2 ? 3 : 2;
-  const float fix_scale = g.order == 2 ? 8388608.0f : 2097152.0f;
-  const float fix_inv = 1.0f / fix_scale;
   if (threadIdx.x < 3) {
     bmin[threadIdx.x] = 1 << 30;
     bmax[threadIdx.x] = -1;
   }
+  if (kDipole && threadIdx.x == 0) wmax = 0ull;
   __syncthreads();
   int lmin[3] = {1 << 30, 1 << 30, 1 << 30}, lmax[3] = {-1, -1, -1};
-#pragma unroll
-  for (int k = 0; k < kDepItems; ++k) {
-    const uint32_t i = b0 + k * kDepThreads + threadIdx.x;
+  double wb = 0.0;
+  for (int k = 0; k < items; ++k) {
+    const uint32_t i = first + k * stride;
     if (i < N) {
       Axis<T> ax[3];
       particle_axes(g, recm, i, ax);
@@ -279,27 +299,51 @@ __global__ void __launch_bounds__(kDepThreads)
         lmin[d] = min(lmin[d], ax[d].c);
         lmax[d] = max(lmax[d], ax[d].c + S - 1);
       }
+      if (kDipole) {
+        const long long idx = orig_index(recp, i);
+        double a = 0.0;
+        for (int d = 0; d < 3; ++d) a += fabs(w[3 * idx + d] * g.inv_h[d]);
+        wb = a > wb || !(a == a) ? a : wb;
+      }
     }
   }
   for (int d = 0; d < 3; ++d) {
-    int a = lmin[d], b = lmax[d];
-    for (int o = 16; o > 0; o >>= 1) {
-      a = min(a, __shfl_xor_sync(0xffffffffu, a, o));
-      b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-    }
+    const int a = __reduce_min_sync(0xffffffffu, lmin[d]);
+    const int b = __reduce_max_sync(0xffffffffu, lmax[d]);
     if ((threadIdx.x & 31) == 0) {
       atomicMin(&bmin[d], a);
       atomicMax(&bmax[d], b);
     }
   }
+  if (kDipole) atomicMax(&wmax, static_cast<unsigned long long>(__double_as_longlong(wb)));
   __syncthreads();
   const int ex = bmax[0] - bmin[0] + 1, ey = bmax[1] - bmin[1] + 1, ez = bmax[2] - bmin[2] + 1;
-  const bool use_tile = static_cast<long long>(ex) * ey * ez <= kTile;
+  bool use_tile = static_cast<long long>(ex) * ey * ez <= kDepTile;
+  // value of the leading word's unit: 2^-21 for charges, whose weights lie in [0, 1] (2^-22 and
+  // 2^-21 for FP32: at most 27/64 with TSC, 1 with CIC); 2^(e - 19) for dipoles, 2^e above wmax
+  double unit = 1.0 / 2097152.0;
+  if constexpr (kDipole) {
+    const int e = static_cast<int>(wmax >> 52) - 1022;  // (the bits of a non-negative double)
+    // not finite, or too large or small for T's scaled products
+    if (e > kMaxExp || (e < -kMaxExp && wmax != 0ull)) use_tile = false;
+    unit = use_tile && wmax != 0ull
+               ? __longlong_as_double(static_cast<long long>(e - 19 + 1023) << 52)
+               : 1.0;
+  } else if (kWords == 1 && g.order == 2) {
+    unit = 1.0 / 8388608.0;
+  }
   if (use_tile)
-    for (int t = threadIdx.x; t < ex * ey * ez; t += kDepThreads) tile[t] = Slot(0);
+    for (int t = threadIdx.x; t < ex * ey * ez; t += kDepThreads)
+#pragma unroll
+      for (int q = 0; q < kWords; ++q) tile[q * kDepTile + t] = 0u;
   __syncthreads();
-  for (int k = 0; k < kDepItems; ++k) {
-    const uint32_t i = b0 + k * kDepThreads + threadIdx.x;
+  // units of the last word per unit of weight (a power of two, multiplied into the z weights once;
+  // 1 where the weights go to the mesh themselves)
+  const T scale = use_tile ? static_cast<T>((kWords == 1 ? 1.0 : kWords == 2 ? 2097152.0
+                                                                             : 4398046511104.0) / unit)
+                           : T(1);
+  for (int k = 0; k < items; ++k) {
+    const uint32_t i = first + k * stride;
     if (i >= N) continue;
     Axis<T> A[3];
     particle_axes(g, recm, i, A);
@@ -308,35 +352,76 @@ __global__ void __launch_bounds__(kDepThreads)
       const long long idx = orig_index(recp, i);
       for (int d = 0; d < 3; ++d) wv[d] = static_cast<T>(w[3 * idx + d] * g.inv_h[d]);
     }
-    for (int c = 0; c < S; ++c)
-      for (int b = 0; b < S; ++b)
-        for (int a = 0; a < S; ++a) {
-          T v;
-          if (kDipole)
-            v = wv[0] * A[0].dw[a] * A[1].w[b] * A[2].w[c] +
-                wv[1] * A[0].w[a] * A[1].dw[b] * A[2].w[c] +
-                wv[2] * A[0].w[a] * A[1].w[b] * A[2].dw[c];
-          else
-            v = A[0].w[a] * A[1].w[b] * A[2].w[c];
-          const int gx = A[0].c + a, gy = A[1].c + b, gz = A[2].c + c;
-          if (use_tile) {
-            Slot* slot = &tile[((gz - bmin[2]) * ey + (gy - bmin[1])) * ex + (gx - bmin[0])];
-            if constexpr (kFixed)
-              atomicAdd(slot, __float2uint_rn(static_cast<float>(v) * fix_scale));
-            else
-              atomicAdd(slot, v);
-          } else
-            atomicAdd(qpad + real_index(g, gx, gy, gz), v);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      A[2].w[c] *= scale;
+      A[2].dw[c] *= scale;
+    }
+    // one row of nodes along x, at the weights (wb, db) of the y and (wc, dc) of the z node
+    auto row = [&](int b, int c, T wb, T db, T wc, T dc) {
+      const T wyz = wb * wc;
+      const T dyz = db * wc, ydz = wb * dc;
+      const int gy = A[1].c + b, gz = A[2].c + c;
+      uint32_t* slot = tile + ((gz - bmin[2]) * ey + (gy - bmin[1])) * ex + (A[0].c - bmin[0]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (a >= S) break;
+        T v;
+        if (kDipole)
+          v = wv[0] * A[0].dw[a] * wyz + A[0].w[a] * (wv[1] * dyz + wv[2] * ydz);
+        else
+          v = A[0].w[a] * wyz;
+        if (use_tile) {
+          if constexpr (kWords == 1) {
+            atomicAdd(slot + a, __float2uint_rn(static_cast<float>(v)));
+          } else if constexpr (kWords == 2) {
+            const long long q = __float2ll_rn(static_cast<float>(v));
+            atomicAdd(slot + a, static_cast<uint32_t>(q >> 21));
+            atomicAdd(slot + a + kDepTile, static_cast<uint32_t>(q) & 0x1fffffu);
+          } else {
+            const long long q = __double2ll_rn(v);
+            atomicAdd(slot + a, static_cast<uint32_t>(q >> 42));
+            atomicAdd(slot + a + kDepTile, static_cast<uint32_t>(q >> 21) & 0x1fffffu);
+            atomicAdd(slot + a + 2 * kDepTile, static_cast<uint32_t>(q) & 0x1fffffu);
+          }
+        } else {
+          atomicAdd(qpad + real_index(g, A[0].c + a, gy, gz), v);
         }
+      }
+    };
+    if constexpr (kShare) {
+      auto pick = [](const T (&v)[3], int k) { return k == 0 ? v[0] : (k == 1 ? v[1] : v[2]); };
+      for (int cb = part; cb < S * S; cb += kShareLanes) {
+        const int c = cb / S, b = cb - c * S;
+        row(b, c, pick(A[1].w, b), pick(A[1].dw, b), pick(A[2].w, c), pick(A[2].dw, c));
+      }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+          if (c < S && b < S) row(b, c, A[1].w[b], A[1].dw[b], A[2].w[c], A[2].dw[c]);
+    }
   }
   if (!use_tile) return;
   __syncthreads();
   for (int t = threadIdx.x; t < ex * ey * ez; t += kDepThreads) {
     T v;
-    if constexpr (kFixed)
-      v = static_cast<T>(static_cast<float>(tile[t]) * fix_inv);
-    else
-      v = tile[t];
+    if constexpr (kWords == 1) {
+      v = static_cast<float>(tile[t]) * static_cast<float>(unit);
+    } else {
+      // the leading word is signed for dipoles; the words' sums overlap, so they join as integers
+      const long long hi = kDipole ? static_cast<long long>(static_cast<int32_t>(tile[t]))
+                                   : static_cast<long long>(tile[t]);
+      if constexpr (kWords == 2) {
+        const long long q = (hi << 21) + static_cast<long long>(tile[kDepTile + t]);
+        v = static_cast<T>(static_cast<double>(q) * (unit / 2097152.0));
+      } else {
+        const unsigned long long mid = tile[kDepTile + t], low = tile[2 * kDepTile + t];
+        v = static_cast<T>((static_cast<double>(hi) * unit) +
+                           static_cast<double>((mid << 21) + low) * (unit / 4398046511104.0));
+      }
+    }
     if (v != T(0)) {
       const int gx = bmin[0] + t % ex, gy = bmin[1] + (t / ex) % ey, gz = bmin[2] + t / (ex * ey);
       atomicAdd(qpad + real_index(g, gx, gy, gz), v);
@@ -984,22 +1069,32 @@ void launch_det_sum_mesh(const p3m_ctx* c) {
   k_det_combine<<<1, kThreads, 0, c->work>>>(c->dred + kDetBlocks, c->energy_acc + 1);
 }
 
+// The block shape for n particles (kDepManyParticles, kDepLanesBelow).
+template <typename T, bool kDipole>
+void run_deposit(const p3m_ctx* c, int64_t n, const double* w) {
+  const int items = n >= kDepManyParticles ? kDepItems : 1;
+  const bool share = n < kDepLanesBelow;
+  const int64_t per_block = static_cast<int64_t>(kDepThreads / (share ? kShareLanes : 1)) * items;
+  constexpr size_t smem = sizeof(uint32_t) * dep_words<T, kDipole>() * dep_tile<T>();
+  auto kern = share ? k_deposit_tiled<T, kDipole, true> : k_deposit_tiled<T, kDipole, false>;
+  if (smem >= 48 * 1024)  // (a few static bytes come on top)
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  using Rec = typename RecT<T>::type;
+  const Rec* rec = static_cast<const Rec*>(sizeof(T) == 4 ? c->recp : c->recm);
+  kern<<<static_cast<unsigned>((n + per_block - 1) / per_block), kDepThreads, smem, c->work>>>(
+      c->g, c->starts + c->nkeys, rec, rec, w, static_cast<T*>(c->qpad), items);
+}
+
 void launch_deposit(const p3m_ctx* c, int64_t n) {
   if (c->det) {
     launch_deposit_det(c, n, nullptr);
     return;
   }
   if (n == 0) return;
-  const uint32_t* total = c->starts + c->nkeys;
-  const unsigned blocks = static_cast<unsigned>((n + kDepPerBlock - 1) / kDepPerBlock);
   if (c->fp32)
-    k_deposit_tiled<float, false><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const float4*>(c->recp), static_cast<const float4*>(c->recp),
-        nullptr, static_cast<float*>(c->qpad));
+    run_deposit<float, false>(c, n, nullptr);
   else
-    k_deposit_tiled<double, false><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recm),
-        nullptr, static_cast<double*>(c->qpad));
+    run_deposit<double, false>(c, n, nullptr);
 }
 
 void launch_dipole_deposit(const p3m_ctx* c, int64_t n, const double* w) {
@@ -1008,16 +1103,10 @@ void launch_dipole_deposit(const p3m_ctx* c, int64_t n, const double* w) {
     return;
   }
   if (n == 0) return;
-  const uint32_t* total = c->starts + c->nkeys;
-  const unsigned blocks = static_cast<unsigned>((n + kDepPerBlock - 1) / kDepPerBlock);
   if (c->fp32)
-    k_deposit_tiled<float, true><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const float4*>(c->recp), static_cast<const float4*>(c->recp), w,
-        static_cast<float*>(c->qpad));
+    run_deposit<float, true>(c, n, w);
   else
-    k_deposit_tiled<double, true><<<blocks, kDepThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const Rec64*>(c->recm), w,
-        static_cast<double*>(c->qpad));
+    run_deposit<double, true>(c, n, w);
 }
 
 void launch_green_multiply(const p3m_ctx* c, bool want_phi, bool want_diff, bool want_energy) {

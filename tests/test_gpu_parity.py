@@ -7,6 +7,8 @@ in-cutoff pair count is an integer decided in FP64 on both sides and must match 
 import dataclasses
 import math
 
+import itertools
+
 import numpy as np
 import pytest
 import torch
@@ -864,3 +866,54 @@ def test_fp32_dense_tiles(n, rows):
     assert rel(ctx.forces(cuda(x)), ref.F) <= TOL[1]
     ctx.sync()
     ctx.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("n", [33, 149999, 150000, 600001])
+def test_deposit_block_shapes(n, order, precision):
+    # the charge deposit's block shapes (eight lanes a particle, one particle a lane, four) on both
+    # sides of every change, with 2000 particles on one node among them: the node charges against
+    # sums in extended precision (an FP64 sum of 2000 terms is itself off by up to 2000 roundings),
+    # FP64 to 1e-14 of the largest (63-bit sums inside a block, then FP64 additions), FP32 to 1e-6
+    r = np.random.default_rng(n + order)
+    x = r.uniform(-1e-3, 1e-3, size=(n, 3))
+    P = O.auto_mesh(np.array([[-1e-3] * 3, [1e-3] * 3]), 32, rc_over_h=0.5, assign_order=order)
+    if n > 4000:
+        x[:2000] = np.asarray(P.lo) + 9.0 * np.asarray(P.h)
+    sx = (x - np.asarray(P.lo)) / np.asarray(P.h)
+    c = np.floor(sx + 0.5) if order == 2 else np.floor(sx)
+    u = (sx - c).astype(np.longdouble)
+    wt = [0.5 * (0.5 - u) ** 2, 0.75 - u ** 2, 0.5 * (0.5 + u) ** 2] if order == 2 else [1 - u, u]
+    c = c.astype(np.int64) - (order - 1)
+    Q = np.zeros(P.n[::-1], dtype=np.longdouble)
+    for i, j, k in itertools.product(range(order + 1), repeat=3):
+        np.add.at(Q, (c[:, 2] + k, c[:, 1] + j, c[:, 0] + i), wt[i][:, 0] * wt[j][:, 1] * wt[k][:, 2])
+    Q = Q * P.q
+    ctx = p3m().Context(gpu_params(P, precision), n)
+    ctx.deposit(cuda(x))
+    q = ctx.get_mesh(0).cpu().numpy()
+    ctx.sync()
+    ctx.close()
+    assert np.abs(q - Q).max() <= (1e-14 if precision == 0 else 1e-6) * np.abs(Q).max()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e-200, 1e60])
+def test_vjp_weight_magnitudes(scale, precision):
+    # the dipole deposit's fixed-point blocks and the FP64 short range's scaled weights: a product
+    # is linear in w whatever w's magnitude, also where half of the weights are zero or 1e-6 of the
+    # rest (FP32: magnitudes that FP32 holds)
+    if precision == 1 and not 1e-31 < scale < 1e9:
+        pytest.skip("outside FP32's range")
+    x = bunch_4k(True)
+    P = O.auto_mesh(x, 16, rc_over_h=2.0, pm_bc=1, pp_bc=1, z_cathode=0.0)
+    w = np.random.default_rng(3).standard_normal(x.shape)
+    w[::2] = 0.0
+    w[1::4] *= 1e-6
+    ref = O.force_vjp(x, w, P)
+    ctx = p3m().Context(gpu_params(P, precision), len(x))
+    g = ctx.force_vjp(cuda(x), cuda(w * scale))
+    ctx.sync()
+    ctx.close()
+    assert rel(g / scale, ref) <= (1e-11 if precision == 0 else 2e-5)
