@@ -30,42 +30,6 @@ namespace {
 
 constexpr int kThreads = 128;
 
-// Calls visit(j0, j1) for every neighbour row of the query point (px, py, pz) (cutoff units)
-// that can hold particles within distance 1, with [j0, j1) the sorted range of its cells whose
-// x-extent meets (px - w, px + w), w = sqrt(1 - d^2) + slack, d the point's distance to the
-// row's (y, z) rectangle less the slack. The slack (Geom::slack) exceeds every rounding in where
-// the sort placed a particle, so no particle within distance 1 is left out.
-template <typename T, typename V>
-__device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restrict__ starts, T px,
-                                         T py, T pz, int part, int parts, V&& visit) {
-  const T slack = static_cast<T>(g.slack);
-  const T cwy = static_cast<T>(g.cw[1]), cwz = static_cast<T>(g.cw[2]);
-  const T iwx = static_cast<T>(g.inv_cw[0]), iwy = static_cast<T>(g.inv_cw[1]),
-          iwz = static_cast<T>(g.inv_cw[2]);
-  const int y0 = max(static_cast<int>(floor((py - T(1) - slack) * iwy)), 0);
-  const int y1 = min(static_cast<int>(floor((py + T(1) + slack) * iwy)), g.nc[1] - 1);
-  const int z0 = max(static_cast<int>(floor((pz - T(1) - slack) * iwz)), 0);
-  const int z1 = min(static_cast<int>(floor((pz + T(1) + slack) * iwz)), g.nc[2] - 1);
-  int turn = 0;
-  for (int rz = z0; rz <= z1; ++rz) {
-    const T zl = static_cast<T>(rz) * cwz, zh = zl + cwz;
-    const T dz = max((pz < zl ? zl - pz : (pz > zh ? pz - zh : T(0))) - slack, T(0));
-    for (int ry = y0; ry <= y1; ++ry) {
-      if ((turn++ & (parts - 1)) != part) continue;
-      const T yl = static_cast<T>(ry) * cwy, yh = yl + cwy;
-      const T dy = max((py < yl ? yl - py : (py > yh ? py - yh : T(0))) - slack, T(0));
-      const T d2 = dy * dy + dz * dz;
-      if (d2 >= T(1)) continue;
-      const T w = sqrt(T(1) - d2) + slack;
-      const int c0 = max(static_cast<int>(floor((px - w) * iwx)), 0);
-      const int c1 = min(static_cast<int>(floor((px + w) * iwx)), g.nc[0] - 1);
-      if (c0 > c1) continue;
-      const uint32_t base = (static_cast<uint32_t>(rz) * g.nc[1] + ry) * g.nc[0];
-      visit(starts[base + c0], starts[base + c1 + 1]);
-    }
-  }
-}
-
 // ------------------------------------------------------------------------------------------
 // FP32 short range: each unordered pair once (Newton's third law), each lane holding two
 // particles and walking their candidate lists in lockstep with the other lanes.
@@ -109,7 +73,6 @@ constexpr int kPpBlocksPerSm = 6;    // resident blocks per SM of the short rang
 // 5003 particles 308, 183, 126, 89, 73 us; 131,072 (dense) 3.57, 2.70, 1.88, 1.95, 2.00 ms;
 // 261,121 (sphere) 184, 155, 156, 175, 214 us; 2,097,152 748 us (1), 846, 949 (2, 4).
 constexpr int kPpMaxLogParts = 4;
-constexpr int kVjpBlocksPerSm = 10;  // resident blocks per SM of its adjoint (48 registers)
 
 // pair_poly on the hardware approximations; r2 in (0, 1]
 template <int kDeg>
@@ -563,172 +526,6 @@ __global__ void k_pp_count_f32(Geom g, const uint32_t* __restrict__ total,
   warp_add_u64(n, out);
 }
 
-// ------------------------------------------------------------------------------------------
-// FP32 vector-Jacobian product of the short-range force map, each unordered pair once: for a
-// pair (i, j), j > i, with d = xi_i - xi_j and H(d) = fco(rho) I + dfr(rho) d d^T (the pair
-// energy's Hessian, even in d), i gets H(d) (w_i - w_j) and j gets its negative. Same walk as
-// k_pp_f32 (persistent blocks, runs in shared memory, 256-bit record loads); w in sorted
-// order as float4 (ws). The result goes to acc4 (zeroed, cutoff units); image pairs (pp_bc)
-// act on i only: acc_i -= H(d)(w_i - S w_j), d = xi_i - S xi_j.
-// ------------------------------------------------------------------------------------------
-template <int kDeg>
-__device__ __forceinline__ void pair_hess_poly(const PairPoly& P, float r2, float& fco,
-                                               float& dfr) {
-  const float rinv = rsqrtf(r2);
-  const float rho = r2 * rinv;
-  const float R = erfcx_poly<kDeg, false>(P, rho);
-  const float ex = exp2f(-P.kappa2_log2e * r2);
-  const float pot = R * ex * rinv;           // erfc(kappa rho) / rho
-  const float cex = P.c2k * ex;
-  const float A = pot + cex;                 // rho^2 times the force coefficient
-  const float rinv2 = rinv * rinv;
-  fco = A * rinv2;
-  // dA/drho = -c2k e/rho - erfc/rho^2 - 2 kappa^2 rho c2k e; dfr = (dA/rho^2 - 2 A/rho^3)/rho
-  const float dA = -(cex + pot) * rinv - 2.f * P.kappa2 * rho * cex;
-  dfr = (dA - 2.f * A * rinv) * rinv2 * rinv;
-}
-
-template <int kDeg, int kRows>
-__global__ void __launch_bounds__(kThreads, kVjpBlocksPerSm)
-    k_pp_vjp_f32(Geom g, PairPoly P, const uint32_t* __restrict__ total,
-                 const float4* __restrict__ rec, const uint32_t* __restrict__ starts,
-                 const float4* __restrict__ ws, float4* __restrict__ acc4,
-                 uint32_t* __restrict__ next_tile) {
-  using R = Rows<kRows>;
-  __shared__ uint32_t run_j0[R::half][kThreads], run_j1[R::half][kThreads];
-  __shared__ uint32_t tile_s;
-  const int tid = threadIdx.x;
-  const uint32_t N = *total;
-  for (;;) {
-    if (tid == 0) tile_s = atomicAdd(next_tile, 1u);
-    __syncthreads();
-    const uint32_t tile = tile_s;
-    __syncthreads();
-    if (static_cast<uint64_t>(tile) * kThreads >= N) break;
-    const uint32_t i = tile * kThreads + tid;
-    const bool alive = i < N;
-    const uint32_t ie = alive ? i : 0u;
-    const float4 pi = rec[2 * ie], li = rec[2 * ie + 1];
-    const float4 wi = ws[ie];
-    int cnt = 0;
-    if (alive) {
-      const uint32_t row = __float_as_uint(li.w) & kRowMask;
-      const int cy = static_cast<int>(row % static_cast<uint32_t>(g.nc[1]));
-      const int cz = static_cast<int>(row / static_cast<uint32_t>(g.nc[1]));
-      for (int r = R::first; r < R::last; ++r) {
-        uint32_t j0, j1;
-        row_range<kRows>(g, starts, pi.x, pi.y, pi.z, cy, cz, r, j0, j1);
-        j0 = max(j0, i + 1);
-        if (j0 < j1) {
-          run_j0[cnt][tid] = j0;
-          run_j1[cnt][tid] = j1;
-          ++cnt;
-        }
-      }
-    }
-    uint32_t ptr = 0, end = 0;
-    if (cnt > 0) {
-      ptr = run_j0[0][tid];
-      end = run_j1[0][tid];
-    }
-    int k = 0;
-    Acc2 sum[3];
-    for (int c = 0; c < 3; ++c) sum[c].hi = sum[c].lo = 0.f;
-    float part[3] = {0.f, 0.f, 0.f};
-    auto pair = [&](bool hit, float r2, float rx, float ry, float rz, uint32_t j) {
-      float fco, dfr;
-      pair_hess_poly<kDeg>(P, hit ? r2 : 0.5f, fco, dfr);
-      const float4 wj = ws[hit ? j : ie];
-      const float v0 = wi.x - wj.x, v1 = wi.y - wj.y, v2 = wi.z - wj.z;
-      const float dv = hit ? dfr * (rx * v0 + ry * v1 + rz * v2) : 0.f;
-      fco = hit ? fco : 0.f;
-      const float c0 = fmaf(fco, v0, dv * rx), c1 = fmaf(fco, v1, dv * ry),
-                  c2 = fmaf(fco, v2, dv * rz);
-      part[0] += c0;
-      part[1] += c1;
-      part[2] += c2;
-      if (hit) red_add_v4(acc4 + j, -c0, -c1, -c2, 0.f);
-    };
-    int step = 0;
-    while (__any_sync(0xffffffffu, ptr < end)) {
-      const bool va = ptr < end, vb = ptr + 1 < end;
-      const float4* pa = va ? rec + 2 * static_cast<size_t>(ptr) : rec;
-      const float4* pb = vb ? rec + 2 * static_cast<size_t>(ptr + 1) : rec;
-      float4 ha, la, hb, lb;
-      load_rec32(pa, ha, la);
-      load_rec32(pb, hb, lb);
-      const float ax = (pi.x - ha.x) + (li.x - la.x), ay = (pi.y - ha.y) + (li.y - la.y),
-                  az = (pi.z - ha.z) + (li.z - la.z);
-      const float bx = (pi.x - hb.x) + (li.x - lb.x), by = (pi.y - hb.y) + (li.y - lb.y),
-                  bz = (pi.z - hb.z) + (li.z - lb.z);
-      const float ra = ax * ax + ay * ay + az * az, rb = bx * bx + by * by + bz * bz;
-      const bool hita = va && ra < 1.f && ra > 0.f;
-      const bool hitb = vb && rb < 1.f && rb > 0.f;
-      if (__any_sync(0xffffffffu, hita)) pair(hita, ra, ax, ay, az, ptr);
-      if (__any_sync(0xffffffffu, hitb)) pair(hitb, rb, bx, by, bz, ptr + 1);
-      ptr += 2;
-      {
-        // the next run without a branch: slot k stays in bounds (k < cnt, or k = 0)
-        const bool sw = ptr >= end && k + 1 < cnt;
-        k += sw ? 1 : 0;
-        const uint32_t nj0 = run_j0[k][tid], nj1 = run_j1[k][tid];
-        ptr = sw ? nj0 : ptr;
-        end = sw ? nj1 : end;
-      }
-      if ((++step & 7) == 0) {
-        for (int c = 0; c < 3; ++c) {
-          sum[c].add(part[c]);
-          part[c] = 0.f;
-        }
-      }
-    }
-    for (int c = 0; c < 3; ++c) sum[c].add(part[c]);
-    if (alive && g.pp_bc) {
-      const double zi = static_cast<double>(pi.z) + static_cast<double>(li.z);
-      if (zi - 0.5 * g.img_c < 1.0) {
-        const float mz = static_cast<float>(g.img_c - zi);
-        const float ch = static_cast<float>(g.img_c);
-        const float cl = static_cast<float>(g.img_c - static_cast<double>(ch));
-        for_rows<float>(g, starts, pi.x, pi.y, mz, 0, 1, [&](uint32_t ja, uint32_t jb) {
-          float rowv[3] = {0.f, 0.f, 0.f};
-          for (uint32_t jj = ja; jj < jb; ++jj) {
-            const float4 hj = rec[2 * jj], lj = rec[2 * jj + 1];
-            const float ax = (pi.x - hj.x) + (li.x - lj.x);
-            const float ay = (pi.y - hj.y) + (li.y - lj.y);
-            const float s = pi.z + hj.z;
-            const float bp = s - pi.z;
-            const float e = (pi.z - (s - bp)) + (hj.z - bp);
-            const float az = ((s - ch) + e) + ((li.z + lj.z) - cl);
-            const float r2 = ax * ax + ay * ay + az * az;
-            if (r2 < 1.f && r2 > 0.f) {
-              float fco, dfr;
-              pair_hess_poly<kDeg>(P, r2, fco, dfr);
-              const float4 wj = ws[jj];
-              const float v0 = wi.x - wj.x, v1 = wi.y - wj.y, v2 = wi.z + wj.z;  // w_i - S w_j
-              const float dv = dfr * (ax * v0 + ay * v1 + az * v2);
-              rowv[0] -= fmaf(fco, v0, dv * ax);
-              rowv[1] -= fmaf(fco, v1, dv * ay);
-              rowv[2] -= fmaf(fco, v2, dv * az);
-            }
-          }
-          for (int c = 0; c < 3; ++c) sum[c].add(rowv[c]);
-        });
-      }
-    }
-    if (alive) red_add_v4(acc4 + i, sum[0].value(), sum[1].value(), sum[2].value(), 0.f);
-  }
-}
-
-// w (input order, FP64) -> ws (sorted order, float4): the weights the FP32 VJP pairs read.
-__global__ void k_gather_w(const uint32_t* __restrict__ total, const float4* __restrict__ rec,
-                           const double* __restrict__ w, float4* __restrict__ ws) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= *total) return;
-  const long long idx = __float_as_int(rec[2 * i].w);
-  ws[i] = make_float4(static_cast<float>(w[3 * idx]), static_cast<float>(w[3 * idx + 1]),
-                      static_cast<float>(w[3 * idx + 2]), 0.f);
-}
-
 }  // namespace
 
 void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
@@ -767,10 +564,7 @@ void launch_pp(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
           log_parts, dense, c->energy_acc, c->pair_acc);
     };
     if (c->g.pp_bc) {
-      // every particle less than r_c above the cathode lies in a z row below this cell
-      const double top = (0.5 * c->g.img_c + 1.0 + c->g.slack) * c->g.inv_cw[2];
-      const int rows = std::max(0, std::min(c->g.nc[2], static_cast<int>(std::floor(top)) + 1));
-      const uint32_t near_cell = static_cast<uint32_t>(rows) * c->g.nc[1] * c->g.nc[0];
+      const uint32_t near_cell = near_cathode_cell(c);
       const unsigned iblocks = static_cast<unsigned>(std::min<int64_t>(
           (n * kImgLanes + kThreads - 1) / kThreads, static_cast<int64_t>(c->num_sms) * 8));
       auto images = [&](auto kern) {
@@ -818,6 +612,9 @@ void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaS
   if (!c->fp32) return;  // FP64: the short range counts as it walks
   cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
   if (n == 0) return;
+  // the tiles of the last sort, whatever call it was made for
+  cudaMemsetAsync(c->pp_tile + 1, 0, sizeof(uint32_t), s);
+  launch_dense_tiles(c, n, s);
   const int64_t lane_pairs = (n + 1) / 2;
   auto kern = c->g.rows == 1   ? k_pp_count_f32<1>
               : c->g.rows == 2 ? k_pp_count_f32<2>
@@ -826,46 +623,6 @@ void launch_pp_count(const p3m_ctx* c, int64_t n, unsigned long long* out, cudaS
       c->g, c->starts + c->nkeys, static_cast<const float4*>(c->recp), c->starts,
       dense_flags(c, n), out);
   launch_pp_dense_count(c, n, out, s);
-}
-
-void launch_pp_vjp(const p3m_ctx* c, int64_t n, const double* w, cudaStream_t s) {
-  if (n == 0) return;
-  if (!c->fp32) {
-    launch_pp64_vjp(c, n, w, s);
-    return;
-  }
-  const unsigned blocks = static_cast<unsigned>((n + kThreads - 1) / kThreads);
-  const uint32_t* total = c->starts + c->nkeys;
-  {
-    // weights in sorted order (in acc, free until the mesh gather), result in fpp (cutoff
-    // units; the mesh gather scales it)
-    float4* ws = reinterpret_cast<float4*>(c->acc);
-    k_gather_w<<<blocks, kThreads, 0, s>>>(total, static_cast<const float4*>(c->recp), w, ws);
-    cudaMemsetAsync(c->fpp, 0, sizeof(float4) * static_cast<size_t>(n), s);
-    cudaMemsetAsync(c->pp_tile, 0, sizeof(uint32_t), s);
-    const unsigned wblocks = static_cast<unsigned>(
-        std::min<int64_t>(blocks, static_cast<int64_t>(kVjpBlocksPerSm) * c->num_sms));
-    auto run = [&](auto k_rows1, auto k_rows2, auto k_rows3) {
-      auto kern = c->g.rows == 1 ? k_rows1 : (c->g.rows == 2 ? k_rows2 : k_rows3);
-      kern<<<wblocks, kThreads, 0, s>>>(c->g, c->poly, total,
-                                        static_cast<const float4*>(c->recp), c->starts, ws,
-                                        static_cast<float4*>(c->fpp), c->pp_tile);
-    };
-    switch (c->poly.deg) {
-      case 4: run(k_pp_vjp_f32<4, 1>, k_pp_vjp_f32<4, 2>, k_pp_vjp_f32<4, 3>); break;
-      case 5: run(k_pp_vjp_f32<5, 1>, k_pp_vjp_f32<5, 2>, k_pp_vjp_f32<5, 3>); break;
-      case 6: run(k_pp_vjp_f32<6, 1>, k_pp_vjp_f32<6, 2>, k_pp_vjp_f32<6, 3>); break;
-      case 7: run(k_pp_vjp_f32<7, 1>, k_pp_vjp_f32<7, 2>, k_pp_vjp_f32<7, 3>); break;
-      case 8: run(k_pp_vjp_f32<8, 1>, k_pp_vjp_f32<8, 2>, k_pp_vjp_f32<8, 3>); break;
-      case 9: run(k_pp_vjp_f32<9, 1>, k_pp_vjp_f32<9, 2>, k_pp_vjp_f32<9, 3>); break;
-      case 10: run(k_pp_vjp_f32<10, 1>, k_pp_vjp_f32<10, 2>, k_pp_vjp_f32<10, 3>); break;
-      case 11: run(k_pp_vjp_f32<11, 1>, k_pp_vjp_f32<11, 2>, k_pp_vjp_f32<11, 3>); break;
-      case 12: run(k_pp_vjp_f32<12, 1>, k_pp_vjp_f32<12, 2>, k_pp_vjp_f32<12, 3>); break;
-      case 13: run(k_pp_vjp_f32<13, 1>, k_pp_vjp_f32<13, 2>, k_pp_vjp_f32<13, 3>); break;
-      case 14: run(k_pp_vjp_f32<14, 1>, k_pp_vjp_f32<14, 2>, k_pp_vjp_f32<14, 3>); break;
-      default: run(k_pp_vjp_f32<15, 1>, k_pp_vjp_f32<15, 2>, k_pp_vjp_f32<15, 3>); break;
-    }
-  }
 }
 
 }  // namespace p3m

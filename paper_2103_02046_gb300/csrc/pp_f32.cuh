@@ -2,6 +2,9 @@
 // force terms and the fitted erfc(x) e^{x^2}.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
+
 #include "pp_common.cuh"
 
 namespace p3m {
@@ -152,6 +155,50 @@ __device__ __forceinline__ float erfcx_poly(const PairPoly& P, float rho) {
 __device__ __forceinline__ bool in_dense_tile(const uint32_t* __restrict__ flags, uint32_t i) {
   const uint32_t f = flags[i >> 6], k = i & 63u;
   return ((f & 1u) && k < ((f >> 8) & 0xffu)) || ((f & 2u) && k >= ((f >> 16) & 0xffu));
+}
+
+// Calls visit(j0, j1) for every neighbour row of the query point (px, py, pz) (cutoff units)
+// that can hold particles within distance 1, with [j0, j1) the sorted range of its cells whose
+// x-extent meets (px - w, px + w), w = sqrt(1 - d^2) + slack, d the point's distance to the
+// row's (y, z) rectangle less the slack. The slack (Geom::slack) exceeds every rounding in where
+// the sort placed a particle, so no particle within distance 1 is left out.
+template <typename T, typename V>
+__device__ __forceinline__ void for_rows(const Geom& g, const uint32_t* __restrict__ starts, T px,
+                                         T py, T pz, int part, int parts, V&& visit) {
+  const T slack = static_cast<T>(g.slack);
+  const T cwy = static_cast<T>(g.cw[1]), cwz = static_cast<T>(g.cw[2]);
+  const T iwx = static_cast<T>(g.inv_cw[0]), iwy = static_cast<T>(g.inv_cw[1]),
+          iwz = static_cast<T>(g.inv_cw[2]);
+  const int y0 = max(static_cast<int>(floor((py - T(1) - slack) * iwy)), 0);
+  const int y1 = min(static_cast<int>(floor((py + T(1) + slack) * iwy)), g.nc[1] - 1);
+  const int z0 = max(static_cast<int>(floor((pz - T(1) - slack) * iwz)), 0);
+  const int z1 = min(static_cast<int>(floor((pz + T(1) + slack) * iwz)), g.nc[2] - 1);
+  int turn = 0;
+  for (int rz = z0; rz <= z1; ++rz) {
+    const T zl = static_cast<T>(rz) * cwz, zh = zl + cwz;
+    const T dz = max((pz < zl ? zl - pz : (pz > zh ? pz - zh : T(0))) - slack, T(0));
+    for (int ry = y0; ry <= y1; ++ry) {
+      if ((turn++ & (parts - 1)) != part) continue;
+      const T yl = static_cast<T>(ry) * cwy, yh = yl + cwy;
+      const T dy = max((py < yl ? yl - py : (py > yh ? py - yh : T(0))) - slack, T(0));
+      const T d2 = dy * dy + dz * dz;
+      if (d2 >= T(1)) continue;
+      const T w = sqrt(T(1) - d2) + slack;
+      const int c0 = max(static_cast<int>(floor((px - w) * iwx)), 0);
+      const int c1 = min(static_cast<int>(floor((px + w) * iwx)), g.nc[0] - 1);
+      if (c0 > c1) continue;
+      const uint32_t base = (static_cast<uint32_t>(rz) * g.nc[1] + ry) * g.nc[0];
+      visit(starts[base + c0], starts[base + c1 + 1]);
+    }
+  }
+}
+
+// First cell of the sort's order above the z rows that hold the particles less than r_c above the
+// cathode (pp_bc): those are the sorted particles before starts[near_cathode_cell].
+inline uint32_t near_cathode_cell(const p3m_ctx* c) {
+  const double top = (0.5 * c->g.img_c + 1.0 + c->g.slack) * c->g.inv_cw[2];
+  const int rows = std::max(0, std::min(c->g.nc[2], static_cast<int>(std::floor(top)) + 1));
+  return static_cast<uint32_t>(rows) * c->g.nc[1] * c->g.nc[0];
 }
 
 }  // namespace p3m

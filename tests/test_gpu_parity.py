@@ -917,3 +917,43 @@ def test_vjp_weight_magnitudes(scale, precision):
     ctx.sync()
     ctx.close()
     assert rel(g / scale, ref) <= (1e-11 if precision == 0 else 2e-5)
+
+
+@pytest.mark.parametrize("n", [2, 12159, 12160, 97279, 97280, 194560])
+def test_fp32_vjp_lanes(n):
+    # FP32 force VJP: from one lane per particle (194,560 particles and more fill the resident
+    # blocks) to 16 lanes that split its rows, on both sides of the changes, images included
+    r = np.random.default_rng(n)
+    x = r.uniform(-1e-3, 1e-3, size=(n, 3))
+    x[:, 2] += 1.02e-3
+    w = r.standard_normal(x.shape)
+    box = np.array([[-1e-3, -1e-3, 0.0], [1e-3, 1e-3, 2.04e-3]])
+    P = O.auto_mesh(box, 32, rc_over_h=1.0 if n > 20000 else 2.0, pm_bc=1, pp_bc=1, z_cathode=0.0)
+    ref = O.force_vjp(x, w, P)
+    ctx = p3m().Context(gpu_params(P, 1), n)
+    g = ctx.force_vjp(cuda(x), cuda(w))
+    ctx.sync()
+    assert rel(g, ref) <= 2e-5
+    ctx.close()
+
+
+def test_candidate_count_after_other_calls():
+    # the candidates of the last call's records, whatever call sorted them: the tiles of dense
+    # regions are found anew (to 2%: the order inside a cell, and with it which particles share a
+    # lane, varies from sort to sort)
+    r = np.random.default_rng(8)
+    x = cuda(r.normal(scale=3e-4, size=(70001, 3)))
+    y = cuda(r.normal(scale=6e-4, size=(70001, 3)))
+    P = O.auto_mesh(np.array([[-3e-3] * 3, [3e-3] * 3]), 32, rc_over_h=2.0)
+    ctx = p3m().Context(gpu_params(P, 1), 70001)
+    ctx.forces(x)
+    want = ctx.candidate_count()
+    ctx.forces(y)
+    assert abs(ctx.candidate_count() - want) > 0.5 * want
+    ctx.force_vjp(x, torch.ones_like(x))
+    assert abs(ctx.candidate_count() - want) <= 0.02 * want
+    ctx.forces(y)
+    ctx.deposit(x)
+    assert abs(ctx.candidate_count() - want) <= 0.02 * want
+    ctx.sync()
+    ctx.close()
