@@ -387,9 +387,12 @@ __global__ void k_dense_count(Geom g, const uint32_t* __restrict__ ntiles,
 
 }  // namespace
 
-// Fewer particles make too few tiles and rows to fill the SMs, and the walk's lanes share them out
-// better (5003 particles: 56 us by the walk, 84 us with tiles).
-constexpr int64_t kDenseMin = 32768;
+// Up to 65,536 particles the walk keeps all of them. Few particles make too few tiles and rows to fill
+// the SMs, and the walk's lanes share them out better (5003 particles: 56 us by the walk, 84 us with
+// tiles); and where particles are few, runs that are differentiated and summed up to a scalar show
+// the other order of summation: the emittance of 60,000 particles after ten steps moved by 5e-9 of its
+// value with tiles.
+constexpr int64_t kDenseMin = 65537;
 
 const uint32_t* dense_flags(const p3m_ctx* c, int64_t n) {
   return n >= kDenseMin ? c->dense_flags : nullptr;

@@ -829,7 +829,7 @@ def test_fp32_lanes_sharing_a_pair(n):
     ctx.close()
 
 
-@pytest.mark.parametrize("n", [32767, 32768, 33001])
+@pytest.mark.parametrize("n", [65536, 65537, 66001])
 @pytest.mark.parametrize("rows", [1, 2, 3])
 def test_fp32_dense_tiles(n, rows):
     # FP32 short range with dense and sparse regions in one bunch, on both sides of the count from
