@@ -16,7 +16,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libp3m.so")
-SOURCES = ["ctx.cu", "sort.cu", "pm.cu", "zconv.cu", "zsolve_df.cu", "box.cu", "pp.cu",
+SOURCES = ["ctx.cu", "sort.cu", "pm.cu", "zconv.cu", "zsolve_df.cu", "fftxy.cu", "box.cu", "pp.cu",
            "pp64.cu", "pp_dense.cu", "pp_vjp.cu", "particles.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

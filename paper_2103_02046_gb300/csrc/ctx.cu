@@ -387,8 +387,9 @@ cufftResult fft_c2r(p3m_ctx* c, void* spec, void* real) {
 }
 
 // Solve on the current qpad: FP64 -> potential; FP32 -> difference fields (and the potential
-// when want_phi).
-p3m_status mesh_solve(p3m_ctx* c, bool want_phi, bool want_diff, bool want_energy) {
+// when want_phi). dipoles: the mesh holds dipoles of weights whose bound is in wbound.
+p3m_status mesh_solve(p3m_ctx* c, bool want_phi, bool want_diff, bool want_energy,
+                      bool dipoles = false) {
   if (c->g.pm_bc == 2) {  // grounded box (FP64): the potential, on the interior nodes
     const p3m_status s = box_solve(c, want_energy);
     if (s != P3M_OK) return fail(c, s, "grounded-box solve failed");
@@ -413,12 +414,16 @@ p3m_status mesh_solve(p3m_ctx* c, bool want_phi, bool want_diff, bool want_energ
   if (c->zsolve_df) {
     // FP64 potential: x-y transforms of the charged planes, the fused z solve in double-float,
     // x-y inverses of the planes z < n_z
-    if (cufftExecD2Z(c->plan_xy_f, static_cast<cufftDoubleReal*>(c->qpad),
-                     static_cast<cufftDoubleComplex*>(c->qhat)) != CUFFT_SUCCESS)
+    if (c->fftxy)
+      launch_fftxy_forward(c, dipoles);
+    else if (cufftExecD2Z(c->plan_xy_f, static_cast<cufftDoubleReal*>(c->qpad),
+                          static_cast<cufftDoubleComplex*>(c->qhat)) != CUFFT_SUCCESS)
       return fail(c, P3M_ECUFFT, "cuFFT forward transform failed");
     launch_zsolve_df(c, want_energy);
-    if (cufftExecZ2D(c->plan_xy_i, static_cast<cufftDoubleComplex*>(c->phihat),
-                     static_cast<cufftDoubleReal*>(c->phireal)) != CUFFT_SUCCESS)
+    if (c->fftxy)
+      launch_fftxy_inverse(c, dipoles);
+    else if (cufftExecZ2D(c->plan_xy_i, static_cast<cufftDoubleComplex*>(c->phihat),
+                          static_cast<cufftDoubleReal*>(c->phireal)) != CUFFT_SUCCESS)
       return fail(c, P3M_ECUFFT, "cuFFT inverse transform failed");
     c->phi_valid = true;
     return P3M_OK;
@@ -492,7 +497,7 @@ p3m_status vjp_impl(p3m_ctx* c, const double* x, int64_t n, const double* w, dou
   launch_vjp_gather(c, n, 0, w, out);
   launch_zero_block(c);
   launch_dipole_deposit(c, n, w);
-  s = mesh_solve(c, false, true, false);
+  s = mesh_solve(c, false, true, false, true);
   if (s != P3M_OK) return s;
   launch_vjp_gather(c, n, 1, w, out);
   c->deposited = false;  // the mesh now holds the dipole deposit
@@ -767,6 +772,7 @@ p3m_status p3m_create(const p3m_params* params, int64_t n_max, void* stream, p3m
     e = zsolve_df_setup(c);
     c->zsolve_df = e == cudaSuccess;
   }
+  if (e == cudaSuccess && fftxy_supported(c)) e = fftxy_setup(c);
   if (e != cudaSuccess) {
     free_all(c);
     delete c;

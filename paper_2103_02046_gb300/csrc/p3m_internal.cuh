@@ -185,6 +185,18 @@ __host__ __device__ inline size_t real_index(const Geom& g, int x, int y, int z)
   return (static_cast<size_t>(z) * g.M[1] + y) * g.M[0] + x;
 }
 
+// The power of two that brings the largest |w| to [1, 4), and its inverse; 1 where no weight is
+// positive and finite.
+__device__ __forceinline__ int w_exponent(unsigned long long bound) {
+  const int e = static_cast<int>((bound >> 52) & 0x7ffull) - 1023;
+  return (bound == 0ull || e == 1024) ? 0 : max(-1000, min(e, 1021));
+}
+__device__ __forceinline__ double w_pow2(int e) {
+  return __longlong_as_double(static_cast<long long>(e + 1023) << 52);
+}
+__device__ __forceinline__ double w_scale(unsigned long long b) { return w_pow2(-w_exponent(b)); }
+__device__ __forceinline__ double w_unscale(unsigned long long b) { return w_pow2(w_exponent(b)); }
+
 __host__ __device__ inline uint32_t pack_node(int cx, int cy, int cz) {
   return static_cast<uint32_t>(cx) | (static_cast<uint32_t>(cy) << 10) |
          (static_cast<uint32_t>(cz) << 20);
@@ -285,7 +297,8 @@ struct p3m_ctx {
   void* phireal = nullptr;      // potential on the doubled mesh
   float2* dfac = nullptr;       // FP32: difference factors e^{2 pi i k/M} - 1 per axis (Mx/2+1 + My + Mz)
   float2* ztw = nullptr;        // fused z solve: e^{-2 pi i t / Mz}, t < Mz (FP32 path: float2;
-                                // FP64 path: double-float, two float2 per entry)
+                                // FP64 path: tables of Mz, Mx and My in double-float, two float2
+                                // per entry, then those of Mx and My in FP64)
   // grounded box (pm_bc = 2, FP64): odd extension (2(n-1))^3, its half spectrum, multiplier
   double* box_real = nullptr;
   double2* box_spec = nullptr;
@@ -294,6 +307,7 @@ struct p3m_ctx {
   bool have_box_f = false, have_box_i = false;
   bool zconv = false;           // FP32 forces use the fused z solve
   bool zsolve_df = false;       // the FP64 potential uses the double-float fused z solve
+  bool fftxy = false;           // and the x and y transforms of fftxy.cu around it
   // Pruned transforms of the doubled mesh: the charge is non-zero, and the fields are needed,
   // only in the n^3 block, so the x-y plane transforms run on the first n_z planes only and
   // the z transforms are strided 1D batches over all (kx, ky) columns.
@@ -366,6 +380,13 @@ void launch_zconv(const p3m_ctx* c, bool want_energy);
 bool zsolve_df_supported(const p3m_ctx* c);
 cudaError_t zsolve_df_setup(p3m_ctx* c);
 void launch_zsolve_df(const p3m_ctx* c, bool want_energy);
+// FP64 path, where all three lengths allow it: x and y transforms (fftxy.cu).
+// scaled: the mesh holds dipoles of the weights w; they are brought to O(1) by the power of two
+// that wbound gives, and back on the way out (the double-float spectra have FP32's exponents).
+bool fftxy_supported(const p3m_ctx* c);
+cudaError_t fftxy_setup(p3m_ctx* c);
+void launch_fftxy_forward(const p3m_ctx* c, bool scaled);
+void launch_fftxy_inverse(const p3m_ctx* c, bool scaled);
 // grounded box (pm_bc = 2): discrete-Laplacian solve of the deposit into phireal
 p3m_status box_setup(p3m_ctx* c);
 p3m_status box_solve(p3m_ctx* c, bool want_energy);

@@ -66,18 +66,6 @@ struct Args64 {
   int log_s;
 };
 
-// The power of two that brings the largest |w| to [1, 4), and its inverse; 1 where no weight is
-// positive and finite.
-__device__ __forceinline__ int w_exponent(unsigned long long bound) {
-  const int e = static_cast<int>((bound >> 52) & 0x7ffull) - 1023;
-  return (bound == 0ull || e == 1024) ? 0 : max(-1000, min(e, 1021));
-}
-__device__ __forceinline__ double w_pow2(int e) {
-  return __longlong_as_double(static_cast<long long>(e + 1023) << 52);
-}
-__device__ __forceinline__ double w_scale(unsigned long long b) { return w_pow2(-w_exponent(b)); }
-__device__ __forceinline__ double w_unscale(unsigned long long b) { return w_pow2(w_exponent(b)); }
-
 // The pair function where there is no table (kappa above 6.5): double-float from the fit, or FP64
 // where that does not reach either. f: force coefficient; g: the potential (hess = false) or the
 // Hessian term.

@@ -957,3 +957,39 @@ def test_candidate_count_after_other_calls():
     assert abs(ctx.candidate_count() - want) <= 0.02 * want
     ctx.sync()
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [32, (32, 64, 128), (256, 32, 32), (32, 256, 64), (1024, 32, 32),
+                               (32, 1024, 32), (33, 32, 32), (32, 40, 64)],
+                         ids=lambda n: str(n).replace(" ", ""))
+@pytest.mark.parametrize("pm_bc", [0, 1])
+def test_fp64_mesh_transforms(n, pm_bc):
+    # FP64 potential: every length of the x and y transforms around the fused z solve (doubled
+    # lengths 64 to 2048, another number of columns to a block for each), and meshes whose x or y
+    # goes to cuFFT instead. Double-float values carry 2^-49; some ten roundings along each axis
+    # give up to 3 * 10 * 2^-49 = 5e-14 of the potential's norm.
+    x = bunch_4k(pm_bc == 1)
+    P = O.auto_mesh(x, n, rc_over_h=2.0, pm_bc=pm_bc, z_cathode=0.0)
+    phi = O.solve(O.deposit(x, P)[0], P)
+    ctx = p3m().Context(gpu_params(P, 0), len(x))
+    ctx.forces(cuda(x), parts=2)
+    assert rel(ctx.get_mesh(1), phi) <= 1e-13
+    ctx.sync()
+    ctx.close()
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-30, 1e-200, 1e60])
+def test_fp64_vjp_weight_magnitudes_on_fused_transforms(scale):
+    # the double-float spectra of the dipole mesh have FP32's exponents: the weights are brought to
+    # O(1) by a power of two and back, so that a product stays linear in w at any magnitude
+    x = bunch_4k(True)
+    P = O.auto_mesh(x, 32, rc_over_h=2.0, pm_bc=1, pp_bc=1, z_cathode=0.0)
+    w = np.random.default_rng(3).standard_normal(x.shape)
+    w[::2] = 0.0
+    w[1::4] *= 1e-6
+    ref = O.force_vjp(x, w, P)
+    ctx = p3m().Context(gpu_params(P, 0), len(x))
+    g = ctx.force_vjp(cuda(x), cuda(w * scale))
+    ctx.sync()
+    ctx.close()
+    assert rel(g / scale, ref) <= 1e-11
