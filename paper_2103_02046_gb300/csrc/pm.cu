@@ -17,9 +17,11 @@
 // summation by parts:
 //   sum_a phi_a dw(a) = (1/2 - u) D_{c-1} + (1/2 + u) D_c   (TSC),   = D_c   (CIC).
 // This is the same discrete force; only the rounding moves from phi to its differences.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
+#include "dfft.cuh"
 #include "p3m_internal.cuh"
 
 namespace p3m {
@@ -819,6 +821,106 @@ __global__ void k_interp(Geom g, const uint32_t* __restrict__ total,
   }
 }
 
+// The FP64 path's interpolation in double-float arithmetic. In FP64 it is bound by the two FP64 lanes
+// per clock and SM: 90 multiply-adds over the 27 nodes, the weights, and the sum with the short range.
+// The force needs only differences of the potential, which FP64 subtractions give (27 of them, those
+// along x between neighbours and one per row against the centre node); all that follows is
+// double-float on the FP32 pipes, whose error, 2^-49 of the differences, lies below the rounding of
+// FP64 sums of the potential itself, a few hundred times larger.
+// (2,097,152 particles 469 -> 268 us. Few particles leave both waiting on latency, of which the
+// longer double-float chains have more: 4096 particles 14.5 us in FP64, 18.4 us in double-float.)
+constexpr int64_t kInterpDfMin = 100000;
+
+// One axis: first node, weights w and their derivatives dw in double-float.
+template <int kOrder>
+struct AxisDF {
+  int c;
+  F2 w[kOrder + 1], dw[kOrder + 1];
+};
+
+template <int kOrder>
+__device__ __forceinline__ AxisDF<kOrder> axis_df(int c, double uf) {
+  AxisDF<kOrder> a;
+  const F2 u = dfm::split_double(uf);
+  if constexpr (kOrder == 2) {
+    a.c = c - 1;
+    const F2 l = dadd(F2{0.5f, 0.f}, dfm::neg(u)), r = dadd(F2{0.5f, 0.f}, u);
+    const F2 l2 = dfm::mul(l, l), r2 = dfm::mul(r, r);
+    a.w[0] = F2{0.5f * l2.hi, 0.5f * l2.lo};
+    a.w[1] = dadd(F2{0.75f, 0.f}, dfm::neg(dfm::mul(u, u)));
+    a.w[2] = F2{0.5f * r2.hi, 0.5f * r2.lo};
+    a.dw[0] = dfm::neg(l);
+    a.dw[1] = F2{-2.f * u.hi, -2.f * u.lo};
+    a.dw[2] = r;
+  } else {
+    a.c = c;
+    a.w[0] = dadd(F2{1.f, 0.f}, dfm::neg(u));
+    a.w[1] = u;
+    a.dw[0] = F2{-1.f, 0.f};
+    a.dw[1] = F2{1.f, 0.f};
+  }
+  return a;
+}
+
+// sum over S terms of v[k] w[k]
+template <int S>
+__device__ __forceinline__ F2 dot_df(const F2 (&v)[S], const F2 (&w)[S]) {
+  F2 s = dfm::mul(v[0], w[0]);
+#pragma unroll
+  for (int k = 1; k < S; ++k) s = dadd(s, dfm::mul(v[k], w[k]));
+  return s;
+}
+
+template <int kOrder>
+__global__ void __launch_bounds__(kThreads)
+    k_interp_df(Geom g, const uint32_t* __restrict__ total, const Rec64* __restrict__ recm,
+                const double* __restrict__ phi, D4* __restrict__ fpp, int parts,
+                double pp_scale) {
+  constexpr int S = kOrder + 1;
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= *total) return;
+  const Rec64 rec = recm[i];
+  const uint32_t node = static_cast<uint32_t>(rec.idx);
+  const AxisDF<kOrder> ax = axis_df<kOrder>(static_cast<int>(node & 1023u), rec.u[0]),
+                       ay = axis_df<kOrder>(static_cast<int>((node >> 10) & 1023u), rec.u[1]),
+                       az = axis_df<kOrder>(static_cast<int>(node >> 20), rec.u[2]);
+  constexpr int m = kOrder == 2 ? 1 : 0;  // the centre of a row, and of the rows
+  const double ref = phi[real_index(g, ax.c + m, ay.c + m, az.c + m)];
+  F2 zx[S], zy[S], z0[S];  // per plane: sums over its rows of w sdx, dw sx, w sx
+#pragma unroll
+  for (int c = 0; c < S; ++c) {
+    F2 sx[S], sdx[S];  // per row: sum_a w (phi - ref), sum_a dw phi
+#pragma unroll
+    for (int b = 0; b < S; ++b) {
+      const double* row = phi + real_index(g, ax.c, ay.c + b, az.c + c);
+      const double p = row[m];
+      // the weights sum to 1 and their derivatives to 0
+      const F2 q = dfm::split_double(p - ref);
+      const F2 r = dfm::split_double(row[m + 1] - p);
+      sx[b] = dadd(q, dfm::mul(ax.w[m + 1], r));
+      if constexpr (kOrder == 2) {
+        const F2 l = dfm::split_double(row[0] - p);
+        sx[b] = dadd(sx[b], dfm::mul(ax.w[0], l));
+        sdx[b] = dadd(dfm::mul(ax.dw[2], r), dfm::mul(ax.dw[0], l));
+      } else {
+        sdx[b] = r;
+      }
+    }
+    zx[c] = dot_df<S>(sdx, ay.w);
+    zy[c] = dot_df<S>(sx, ay.dw);
+    z0[c] = dot_df<S>(sx, ay.w);
+  }
+  double F[3] = {g.fscale[0] * d_of(dot_df<S>(zx, az.w)), g.fscale[1] * d_of(dot_df<S>(zy, az.w)),
+                 g.fscale[2] * d_of(dot_df<S>(z0, az.dw))};
+  if (parts & 1) {
+    const D4 s = fpp[i];
+    F[0] += pp_scale * s.x;
+    F[1] += pp_scale * s.y;
+    F[2] += pp_scale * s.z;
+  }
+  fpp[i] = D4{F[0], F[1], F[2], 0.0};
+}
+
 // f[i] = the force of input particle i, gathered from sorted order through its sorted position
 // (keys[i] after the scatter); particles left out of the sort (outside the mesh) get zero.
 template <typename T>
@@ -1137,9 +1239,20 @@ void launch_interp(const p3m_ctx* c, int64_t n, double* f, int parts) {
         pp_scale);
     k_unpermute<float><<<blocks_for(n), kThreads, 0, c->work>>>(c->keys, n, c->fpp, f);
   } else {
-    k_interp<double><<<blocks_for(n), kThreads, 0, c->work>>>(
-        c->g, total, static_cast<const Rec64*>(c->recm), static_cast<const double*>(c->phireal),
-        c->n_real, c->fpp, nullptr, nullptr, parts, static_cast<float>(pp_scale), pp_scale);
+    // the potential's unit has to leave room for N particles and for the low parts of its
+    // differences in FP32's exponents
+    const double unit = c->g.ke * std::fabs(c->g.q) / *std::max_element(c->g.h, c->g.h + 3);
+    const auto* recm = static_cast<const Rec64*>(c->recm);
+    const auto* phi = static_cast<const double*>(c->phireal);
+    if ((parts & 2) && n >= kInterpDfMin && !c->g.force_diff && unit > 1e-18 && unit < 1e25) {
+      auto kern = c->g.order == 2 ? k_interp_df<2> : k_interp_df<1>;
+      kern<<<blocks_for(n), kThreads, 0, c->work>>>(c->g, total, recm, phi,
+                                                    static_cast<D4*>(c->fpp), parts, pp_scale);
+    } else {
+      k_interp<double><<<blocks_for(n), kThreads, 0, c->work>>>(
+          c->g, total, recm, phi, c->n_real, c->fpp, nullptr, nullptr, parts,
+          static_cast<float>(pp_scale), pp_scale);
+    }
     k_unpermute<double><<<blocks_for(n), kThreads, 0, c->work>>>(c->keys, n, c->fpp, f);
   }
 }

@@ -993,3 +993,23 @@ def test_fp64_vjp_weight_magnitudes_on_fused_transforms(scale):
     ctx.sync()
     ctx.close()
     assert rel(g / scale, ref) <= 1e-11
+
+
+@pytest.mark.parametrize("order", [1, 2])
+@pytest.mark.parametrize("n", [99999, 100000, 100001])
+def test_fp64_interpolation_arithmetic(n, order):
+    # the long-range force of many particles is interpolated in double-float from differences of
+    # the potential, that of few in FP64: on both sides of the change, with particles on nodes and,
+    # TSC, on the points where the nearest node changes (CIC's force jumps on its nodes)
+    r = np.random.default_rng(n + order)
+    x = r.uniform(-1e-3, 1e-3, size=(n, 3))
+    P = O.auto_mesh(np.array([[-1e-3] * 3, [1e-3] * 3]), 32, rc_over_h=1.0, assign_order=order)
+    h, lo = np.asarray(P.h), np.asarray(P.lo)
+    x[:64] = lo + h * (r.integers(3, 28, size=(64, 3)) + (0.5 if order == 1 else 0.0))
+    x[64:128] = lo + h * (0.5 + r.integers(3, 28, size=(64, 3)))
+    ref = O.interp(x, O.solve(O.deposit(x, P)[0], P), P)[0]
+    ctx = p3m().Context(gpu_params(P, 0), n)
+    f = ctx.forces(cuda(x), parts=2)
+    ctx.sync()
+    ctx.close()
+    assert rel(f, ref) <= TOL[0]
