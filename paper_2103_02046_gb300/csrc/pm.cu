@@ -990,32 +990,51 @@ __device__ void hess_from_diff(const Geom& g, const float* __restrict__ D, size_
     }
 }
 
+// Second derivatives of the interpolated potential, summed axis by axis as in grad_from_phi: about 150
+// FP64 operations per particle instead of 540 node by node, from differences to the first node (every
+// term's weights sum to zero), which round less than the potential. Whole FP64 products: 4096 particles
+// on 64^3 375 -> 363 us, 262,144 907 -> 815 us, 1,048,576 on 128^3 3.40 -> 3.07 ms.
 __device__ void hess_from_phi(const Geom& g, const double* __restrict__ phi,
                               const Axis<double> ax[3], double H[3][3]) {
-  const int S = g.order == 2 ? 3 : 2;
-  // second derivative of the 1D weights: TSC {1, -2, 1}, CIC 0
-  const double d2[3] = {1.0, -2.0, 1.0};
   const bool tsc = g.order == 2;
-  for (int d = 0; d < 3; ++d)
-    for (int e = 0; e < 3; ++e) H[d][e] = 0.0;
-  for (int c = 0; c < S; ++c)
+  const int S = tsc ? 3 : 2;
+  const double ref = phi[real_index(g, ax[0].c, ax[1].c, ax[2].c)];
+  double h[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // xx, yy, zz, xy, xz, yz
+  for (int c = 0; c < S; ++c) {
+    // sums over the plane's rows: by the y weights w, dw and the second difference, of the row sums
+    // s (w), d (dw) and e (second difference along x)
+    double ws = 0.0, wd = 0.0, we = 0.0, ds = 0.0, dd = 0.0, es = 0.0;
     for (int b = 0; b < S; ++b) {
       const double* row = phi + real_index(g, ax[0].c, ax[1].c + b, ax[2].c + c);
+      double s = 0.0, d = 0.0;
       for (int a = 0; a < S; ++a) {
-        const double p = row[a];
-        if (tsc) {
-          H[0][0] += p * d2[a] * ax[1].w[b] * ax[2].w[c];
-          H[1][1] += p * ax[0].w[a] * d2[b] * ax[2].w[c];
-          H[2][2] += p * ax[0].w[a] * ax[1].w[b] * d2[c];
-        }
-        H[0][1] += p * ax[0].dw[a] * ax[1].dw[b] * ax[2].w[c];
-        H[0][2] += p * ax[0].dw[a] * ax[1].w[b] * ax[2].dw[c];
-        H[1][2] += p * ax[0].w[a] * ax[1].dw[b] * ax[2].dw[c];
+        const double p = row[a] - ref;
+        s = fma(p, ax[0].w[a], s);
+        d = fma(p, ax[0].dw[a], d);
+      }
+      ws = fma(ax[1].w[b], s, ws);
+      wd = fma(ax[1].w[b], d, wd);
+      ds = fma(ax[1].dw[b], s, ds);
+      dd = fma(ax[1].dw[b], d, dd);
+      if (tsc) {  // the 1D weights' second derivative: TSC {1, -2, 1}, CIC 0
+        const double e = (row[0] - row[1]) + (row[2] - row[1]);
+        we = fma(ax[1].w[b], e, we);
+        es = b == 1 ? fma(-2.0, s, es) : es + s;
       }
     }
-  H[1][0] = H[0][1];
-  H[2][0] = H[0][2];
-  H[2][1] = H[1][2];
+    h[3] = fma(ax[2].w[c], dd, h[3]);
+    h[4] = fma(ax[2].dw[c], wd, h[4]);
+    h[5] = fma(ax[2].dw[c], ds, h[5]);
+    if (tsc) {
+      h[0] = fma(ax[2].w[c], we, h[0]);
+      h[1] = fma(ax[2].w[c], es, h[1]);
+      h[2] = c == 1 ? fma(-2.0, ws, h[2]) : h[2] + ws;
+    }
+  }
+  for (int d = 0; d < 3; ++d) H[d][d] = h[d];
+  H[0][1] = H[1][0] = h[3];
+  H[0][2] = H[2][0] = h[4];
+  H[1][2] = H[2][1] = h[5];
 }
 
 template <typename T>
