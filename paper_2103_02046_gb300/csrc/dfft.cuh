@@ -2,7 +2,7 @@
 // in FP64 (CZ). Double-float: every real is an unevaluated sum hi + lo of two FP32 numbers (about 48
 // significant bits), so the butterflies run on GB300's FP32 pipes instead of its scarce FP64 units.
 //
-// Transforms: power-of-two lengths in [64, 2048], radix-8 Stockham autosort passes (then one
+// Transforms: power-of-two lengths in [16, 2048], radix-8 Stockham autosort passes (then one
 // radix-4 or radix-2 pass when the length's logarithm is not a multiple of 3) in shared memory;
 // twiddles from tables computed on the host in extended precision.
 #pragma once
@@ -221,7 +221,7 @@ __device__ __forceinline__ void drun_pass(int R, E* a, int logN, int logp, int i
 }
 
 // Forward transform (sign -1) of a column that is zero in its upper half, or inverse transform
-// (sign +1) of which only the lower half is kept; unnormalised, length 2^logN >= 64.
+// (sign +1) of which only the lower half is kept; unnormalised, length 2^logN >= 16.
 template <bool kForward, typename E>
 __device__ void dcolumn_fft(E* a, int logN, int i0, int tpc, const E* __restrict__ tw) {
   const float sign = kForward ? -1.f : 1.f;

@@ -163,8 +163,6 @@ __global__ void __launch_bounds__(256, 3)
     if (kForward || y < ny) base[static_cast<size_t>(y) * Hx] = A[mine * padN + dpad(y)];
 }
 
-bool length_ok(int N) { return N >= 64 && N <= 2048 && (N & (N - 1)) == 0; }
-
 // tables of e^{-2 pi i t / M} (zsolve_df_setup): Mz, Mx, My in double-float, Mx, My in FP64
 const CD* table_df(const p3m_ctx* c, int axis) {
   return reinterpret_cast<const CD*>(c->ztw) + c->g.M[2] + (axis == 1 ? c->g.M[0] : 0);
@@ -186,8 +184,10 @@ unsigned y_blocks(const p3m_ctx* c) {
 
 }  // namespace
 
+bool fftxy_length(int N) { return N >= 16 && N <= 2048 && (N & (N - 1)) == 0; }
+
 bool fftxy_supported(const p3m_ctx* c) {
-  return c->zsolve_df && length_ok(c->g.M[0]) && length_ok(c->g.M[1]);
+  return c->zsolve_df && fftxy_length(c->g.M[0]) && fftxy_length(c->g.M[1]);
 }
 
 cudaError_t fftxy_setup(p3m_ctx* c) {

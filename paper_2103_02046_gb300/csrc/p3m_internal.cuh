@@ -383,6 +383,7 @@ void launch_zsolve_df(const p3m_ctx* c, bool want_energy);
 // FP64 path, where all three lengths allow it: x and y transforms (fftxy.cu).
 // scaled: the mesh holds dipoles of the weights w; they are brought to O(1) by the power of two
 // that wbound gives, and back on the way out (the double-float spectra have FP32's exponents).
+bool fftxy_length(int N);
 bool fftxy_supported(const p3m_ctx* c);
 cudaError_t fftxy_setup(p3m_ctx* c);
 void launch_fftxy_forward(const p3m_ctx* c, bool scaled);

@@ -11,7 +11,7 @@
 // kx, Hx = Mx/2 + 1; the charge is non-zero only in planes z < n_z <= Mz / 2. With
 // base = Kf Q - Ki Q(-kz) (Ki absent without the cathode), phihat = base.
 //
-// Transforms: power-of-two Mz in [64, 2048], radix-8 Stockham autosort passes (then one radix-4
+// Transforms: power-of-two Mz in [16, 2048], radix-8 Stockham autosort passes (then one radix-4
 // or radix-2 pass when log2 Mz is not a multiple of 3) in shared memory; twiddles from a table
 // computed in extended precision on the host and split into double-float. A block holds
 // C = 2048 / Mz columns (one 8-point butterfly per thread and pass, 256 threads), taken from the whole
@@ -134,8 +134,12 @@ size_t zsolve_df_smem_bytes(int N) {
 }  // namespace
 
 bool zsolve_df_supported(const p3m_ctx* c) {
-  const int N = c->g.M[2];
-  return !c->fp32 && !c->det && c->g.pm_bc != 2 && N >= 64 && N <= 2048 && (N & (N - 1)) == 0;
+  // Lengths below 64 only with the x-y transforms of fftxy.cu (which scale what they pass on into
+  // FP32's exponents): on a 16^3 mesh the solve is then five kernels of a few microseconds instead of
+  // cuFFT's nine and the multiply.
+  const int* M = c->g.M;
+  if (c->fp32 || c->det || c->g.pm_bc == 2 || !fftxy_length(M[2])) return false;
+  return M[2] >= 64 || (fftxy_length(M[0]) && fftxy_length(M[1]));
 }
 
 cudaError_t zsolve_df_setup(p3m_ctx* c) {

@@ -959,13 +959,14 @@ def test_candidate_count_after_other_calls():
     ctx.close()
 
 
-@pytest.mark.parametrize("n", [32, (32, 64, 128), (256, 32, 32), (32, 256, 64), (1024, 32, 32),
+@pytest.mark.parametrize("n", [8, 16, (16, 32, 8), (20, 16, 16), (16, 32, 32), 32,
+                               (32, 64, 128), (256, 32, 32), (32, 256, 64), (1024, 32, 32),
                                (32, 1024, 32), (33, 32, 32), (32, 40, 64)],
                          ids=lambda n: str(n).replace(" ", ""))
 @pytest.mark.parametrize("pm_bc", [0, 1])
 def test_fp64_mesh_transforms(n, pm_bc):
     # FP64 potential: every length of the x and y transforms around the fused z solve (doubled
-    # lengths 64 to 2048, another number of columns to a block for each), and meshes whose x or y
+    # lengths 16 to 2048, another number of columns to a block for each), and meshes whose x or y
     # goes to cuFFT instead. Double-float values carry 2^-49; some ten roundings along each axis
     # give up to 3 * 10 * 2^-49 = 5e-14 of the potential's norm.
     x = bunch_4k(pm_bc == 1)
