@@ -35,10 +35,10 @@ from paper_2103_02046_gb300 import bunches as B  # noqa: E402
 
 METRIC = "P3M force evals/s and PP pair-interactions/s at N=16M, FP32 vs FP64 at stated error"
 FLOPS_PER_PAIR = 37.0  # algorithmic FP32 flops per in-cutoff pair (FFMA = 2, incl. 3 MUFU)
-KERNELS_PER_EVAL = 10  # bin, 3 scan passes, scatter, short range, deposit, fused z solve,
-                       # interpolation, combination in the caller's order (cuFFT's kernels
-                       # not counted)
-# DRAM bytes (read + write) of one k_pp_f32 launch, from ncu captures (dram__bytes_read.sum +
+KERNELS_PER_EVAL = 13  # bin, 3 scan passes, scatter, list of dense tiles, short range (walk and
+                       # tiles), clearing of the mesh, deposit, fused z solve, interpolation,
+                       # combination in the caller's order (cuFFT's kernels not counted)
+# DRAM bytes (read + write) of the short range's main launch, from ncu captures (dram__bytes_read.sum +
 # dram__bytes_write.sum), with the particle count captured and the limiter the capture showed:
 # the 2,097,152-particle sphere on a 128^3 mesh stands in for the 16M sphere (same density; the
 # kernel reads each 32-B record about once from DRAM and its reductions into the coarse (16 B),
@@ -46,15 +46,15 @@ KERNELS_PER_EVAL = 10  # bin, 3 scan passes, scatter, short range, deposit, fuse
 # particle count); the 1M Gaussian is captured at full size. Workloads without a capture of the
 # current kernel report traffic null.
 PP_DRAM = {
-    "sphere16m": dict(bytes=127.666688e6 + 20.851968e6, particles=2097152,
+    "sphere16m": dict(bytes=127.77728e6 + 20.71552e6, particles=2097152,
                       source="k_pp_f32<6, 2> on the 2,097,152-particle sphere (128^3), scaled "
                              "by particle count",
-                      limiter="L1 data pipe 73%, instruction issue 71%, L2 48% (ncu, "
+                      limiter="L1 data pipe 75%, instruction issue 71%, L2 49% (ncu, "
                               "profiles/k_pp_f32_sphere2m_128.md)"),
-    "gauss1m": dict(bytes=71.533568e6 + 0.91648e6, particles=1048576,
-                    source="k_pp_f32<6, 3> on this workload (1,048,576 particles)",
-                    limiter="L1 data pipe 75%, L2 72% (vector reductions), issue 48% "
-                            "(ncu, profiles/k_pp_f32_gauss1m_64.md)"),
+    "gauss1m": dict(bytes=60.036864e6 + 0.268032e6, particles=1048576,
+                    source="k_pp_dense<6, 3> on this workload (1,048,576 particles)",
+                    limiter="instruction issue 71%, FMA pipe 66%, L1 data pipe 64% "
+                            "(ncu, profiles/k_pp_dense_gauss1m_64.md)"),
 }
 
 
@@ -428,7 +428,7 @@ def run_ours(a, rank, world, local_rank):
         "fp64": {"evals_per_s": fp64_evals, "stage_ms": dict(zip(
             ["bin_sort", "short_range", "deposit", "solve", "interp_combine", "total"], t64))},
         "error": {"fp32_vs_fp64_gpu_rel_l2": err32},
-        "roofline": {"bound": "alu", "kernel": "k_pp_f32 (short range)",
+        "roofline": {"bound": "alu", "kernel": "k_pp_f32 and k_pp_dense (short range)",
                      "limiter": cap["limiter"] if cap else None, "achieved": achieved,
                      "peak": fp32_peak, "unit": "TFLOP/s", "frac": achieved / fp32_peak,
                      "traffic": cap["bytes"] / cap["particles"] * N if cap else None,
