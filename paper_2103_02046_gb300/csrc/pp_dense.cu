@@ -14,7 +14,7 @@
 // A tile pays where its boxes are small against r_c: of the pairs met about 0.43 are within r_c at
 // 36,000 neighbours a particle (rows r_c/3 wide), fewer at lower densities, while the walk's runs
 // per particle keep 0.59 to 0.37. k_dense_tiles therefore hands a stretch of 64 particles to the
-// tiles only if its row holds enough of them (kDenseNeighbours), and the walk takes the others:
+// tiles only if its row holds enough of them (kDenseNeighboursMin), and the walk takes the others:
 // every pair belongs to its earlier particle in sorted order, so the two can be mixed freely.
 //
 // Measured, short range: 1,048,576-particle Gaussian 97.1 -> 38.7 ms, 4,194,304-particle core and
@@ -33,21 +33,25 @@ constexpr int kThreads = 128;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBlocksPerSm = 5;
 constexpr uint32_t kTile = 64;
-// (100, 150, 200, 300, 500, 1000, 3000 neighbours: the dense 131,072-particle bunch takes 1.21, 1.22,
-// 1.21, 1.21, 1.23, 1.39, 1.94 ms, the 2,097,152-particle sphere, whose particles have 67, 1.98,
-// 0.86, 0.78, 0.77, 0.76, 0.76 ms for the walk that is left)
-constexpr int kDenseNeighbours = 300;
+// A region goes to the tiles if its particles have 2000 neighbours, or 300 and four times the mean
+// over the mesh's volume. At a uniform density the walk is ahead up to about 2000 (a sphere with
+// r_c = 3h, tiles against the walk: 131,072 particles of 1200 neighbours 918, 819 us; 1,300,003 of 1400
+// 6.6, 5.3 ms; 16,777,216, of whose 226 neighbours chance makes 300 here and there, 23.4, 17.8 ms), while
+// a bunch with a core is best served by tiles throughout (all of more than 300, 1000, 2000 neighbours:
+// four steps of 131,072 dense particles 6.2, 7.3, 8.7 ms; a Gaussian of 150,000 1.01, 1.24, 1.49 ms). The
+// sphere's density is 2.4 times its mesh's mean.
+constexpr float kDenseNeighboursMin = 300.f, kDenseNeighboursMax = 2000.f, kDensePeak = 4.f;
 // pairs closer than this (in units of r_c, squared) are summed term by term
 constexpr float kClose2 = 1.f / 1024.f;
 
 // One thread per stretch of kTile sorted particles. A stretch lies in one cell row or is cut where
 // a second row begins (stretches over three rows or more stay with the walk); each piece becomes a
-// tile if the particles of its row within r_c of its middle stand for at least kDenseNeighbours
+// tile if the particles of its row within r_c of its middle stand for at least `neighbours`
 // neighbours. Pieces begin and end at even offsets, since the walk takes particles in pairs.
 __global__ void k_dense_tiles(Geom g, const uint32_t* __restrict__ total,
                               const float4* __restrict__ rec, const uint32_t* __restrict__ starts,
                               uint32_t* __restrict__ flags, uint2* __restrict__ tiles,
-                              uint32_t* __restrict__ ntiles) {
+                              uint32_t* __restrict__ ntiles, float neighbours) {
   const uint32_t c = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t N = *total;
   const uint32_t i0 = c * kTile;
@@ -72,7 +76,7 @@ __global__ void k_dense_tiles(Geom g, const uint32_t* __restrict__ total,
     const uint32_t in_row = starts[row * nx + c1 + 1] - starts[row * nx + c0];
     // density = in_row rows^2 / 2 (per r_c^3), neighbours = 4 pi / 3 of that
     return 2.0944f * static_cast<float>(g.rows * g.rows) * static_cast<float>(in_row) >=
-           static_cast<float>(kDenseNeighbours);
+           neighbours;
   };
   uint32_t f = (cut0 - i0) << 8 | (cut1 - i0) << 16;
   if (cut0 > i0 && dense(i0, cut0, row0)) {
@@ -401,10 +405,15 @@ const uint32_t* dense_flags(const p3m_ctx* c, int64_t n) {
 void launch_dense_tiles(const p3m_ctx* c, int64_t n, cudaStream_t s) {
   if (n < kDenseMin) return;
   const int64_t stretches = (n + kTile - 1) / kTile;
+  double volume = 1.0;  // of the mesh, in r_c^3
+  for (int d = 0; d < 3; ++d) volume *= (c->g.n[d] - 1) * c->g.a[d];
+  const float mean = static_cast<float>(4.18879 * static_cast<double>(n) / volume);
+  const float neighbours =
+      std::min(std::max(kDensePeak * mean, kDenseNeighboursMin), kDenseNeighboursMax);
   // the tile count was cleared by the sort, as the item counter behind it
   k_dense_tiles<<<static_cast<unsigned>((stretches + kThreads - 1) / kThreads), kThreads, 0, s>>>(
       c->g, c->starts + c->nkeys, static_cast<const float4*>(c->recp), c->starts, c->dense_flags,
-      c->dense_tiles, c->pp_tile + 1);
+      c->dense_tiles, c->pp_tile + 1, neighbours);
 }
 
 void launch_pp_dense(const p3m_ctx* c, int64_t n, cudaStream_t s, bool want_energy) {
