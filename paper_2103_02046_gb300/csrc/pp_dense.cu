@@ -136,8 +136,9 @@ __device__ __forceinline__ float2 two(float v) {
   return r;
 }
 
-// Force coefficient (and the potential) of a pair at r2, on the hardware approximations
-template <int kDeg, bool kPot>
+// Force coefficient (and the potential) of a pair at r2, on the hardware approximations, in the walk's
+// order of operations: the closest pairs, whose force outweighs all others', get the same bits
+template <int kDeg>
 __device__ __forceinline__ float pair_coef(const PairPoly& P, float r2, float& pot) {
   const float rinv = rsqrt_ftz(r2);
   const float t = rcp_ftz(fmaf(P.pk, r2 * rinv, 1.f));
@@ -146,9 +147,8 @@ __device__ __forceinline__ float pair_coef(const PairPoly& P, float r2, float& p
 #pragma unroll
   for (int m = kDeg - 1; m >= 0; --m) R = fmaf(R, u, P.c[m]);
   const float ex = ex2_ftz(-P.kappa2_log2e * r2);
-  const float tr = t * rinv;
-  if constexpr (kPot) pot = R * tr * ex;
-  return fmaf(R, tr, P.c2k) * (ex * (rinv * rinv));
+  pot = R * t * ex * rinv;
+  return fmaf(P.c2k, ex, pot) * (rinv * rinv);
 }
 
 // A warp's item: one tile and one row of its half shell.
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm)
         const bool ha = r2a < 1.f && r2a > 0.f && (!own || jb + m > ia);
         const bool hb = r2b < 1.f && r2b > 0.f && (!own || jb + m > ib);
         float ua = 0.f, ub = 0.f;
-        float ca = pair_coef<kDeg, kPot>(P, r2a, ua), cb = pair_coef<kDeg, kPot>(P, r2b, ub);
+        float ca = pair_coef<kDeg>(P, r2a, ua), cb = pair_coef<kDeg>(P, r2b, ub);
         ca = ha ? ca : 0.f;
         cb = hb ? cb : 0.f;
         if constexpr (kPot) qp += (ha ? ua : 0.f) + (hb ? ub : 0.f);
