@@ -17,7 +17,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module")
-def checker(tmp_path_factory):
+def program(tmp_path_factory):
     gxx = shutil.which("g++")
     if gxx is None:
         pytest.skip("no g++")
@@ -29,8 +29,8 @@ def checker(tmp_path_factory):
 
 
 @pytest.mark.parametrize("kappa", [0.5, 1.0, 3.0, 6.0])
-def test_pair_table_accuracy(checker, kappa):
-    out = subprocess.run([checker, repr(kappa)], check=True, capture_output=True, text=True)
+def test_pair_table_accuracy(program, kappa):
+    out = subprocess.run([program, repr(kappa)], check=True, capture_output=True, text=True)
     r = json.loads(out.stdout)
     assert r["fit"] and max(r["close"]) < 1e-13
     for key, condition in (("fco", 1.5), ("pot", 0.5), ("dfr", 2.5)):
